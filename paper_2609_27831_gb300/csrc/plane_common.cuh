@@ -137,16 +137,16 @@ struct EpiConst {
                       // kfin M_l^{-1} mod m_l, so that the stored value is the
                       // CRT's v_l = (c mod m_l) M_l^{-1} mod m_l (Sec. 4.4)
   int M, N, row, col0, L1, ell;
-  uint16_t* urow;     // u of this modulus, row `row`
+  uint16_t* uell;     // u of this modulus
   int32_t* dbg;
-  bool vec_ok;        // rows of u start 16-byte aligned
 };
 
 // v_l tiles of one epilogue warp through shared memory: two 2 KB buffers of
 // 32 rows x 64 bytes in the 64-byte swizzle (16-byte chunk q of row r at
 // r 64 + 16 (q ^ ((r >> 1) & 3)): the eight rows of a store phase hit eight
 // different bank groups), each written to u by one TMA store.  map is null
-// when u's rows are not 16-byte multiples; then every thread stores its row.
+// when u's rows are not 16-byte multiples; then the warp writes the staged
+// tile row by row (store_tile_rows).
 struct UStage {
   const CUtensorMap* map;
   uint32_t sbuf;      // shared address of the warp's two buffers
@@ -167,11 +167,40 @@ __device__ __forceinline__ EpiConst epi_const(const DevTables& T, const Job& j, 
   e.col0 = col0;
   e.L1 = P.L1;
   e.ell = j.u.ell;
-  e.urow = P.u + (int64_t)j.u.ell * P.upitch + (int64_t)row * P.N;
+  e.uell = P.u + (int64_t)j.u.ell * P.upitch;
   e.dbg = P.dbg_prods;
-  e.vec_ok = (P.N & 7) == 0;
   e.mul = j.last ? barrett32(mc.kfin * __ldg(crt_view(T.crt_pool, P).Minv + j.u.ell), mc.m, mc.mu) : j.kmul;
   return e;
+}
+
+// A staged 32 x 32 tile of v_l (the 64-byte swizzle above) to u where its rows
+// are only 2-byte aligned (N not a multiple of 8: no TMA store can reach
+// them).  Half a warp takes a row, a lane the two values of a staged word, in
+// two 2-byte stores.  What bounds it is the sectors a store instruction
+// touches: two rows here (4 to 6 sectors of 32 bytes), where a thread storing
+// its own row touched 32 (plane GEMMs of 1531 x 1093 x 1777, p = 512: 2.39 ->
+// 1.14 ms, 1.11 with N = 1096 and the TMA store; 64 uneven problems 23.3 -> 9.0
+// ms).  Pairing values into aligned words across lanes (a shuffle, one 4-byte
+// store and the row's two ends on their own) was slower: 1.40 and 11.5 ms.
+static __device__ __noinline__ void store_tile_rows(uint16_t* uell, uint32_t buf, int row0, int col, int M, int N) {
+  const int lane = threadIdx.x & 31, c = lane & 15;
+  const int c0 = col + 2 * c;
+  const bool in0 = c0 < N, in1 = c0 + 1 < N;
+  uint16_t* dst = uell + (int64_t)(row0 + (lane >> 4)) * N + c0;
+#pragma unroll
+  for (int s = 0; s < 16; ++s) {
+    const int r = 2 * s + (lane >> 4);
+    uint32_t w;
+    asm volatile("ld.shared.b32 %0, [%1];"
+                 : "=r"(w)
+                 : "r"(buf + (uint32_t)(r * 64 + 16 * ((c >> 2) ^ (s & 3)) + 4 * (c & 3)))
+                 : "memory");
+    if (row0 + r < M) {
+      if (in0) dst[0] = (uint16_t)w;
+      if (in1) dst[1] = (uint16_t)(w >> 16);
+    }
+    dst += 2 * (int64_t)N;
+  }
 }
 
 // One 32-column chunk of a job's accumulator (v, read from taddr; columns
@@ -198,43 +227,36 @@ __device__ __forceinline__ void epi_chunk(const Job& j, const EpiConst& e, uint3
     if (e.mul != 1u) r = barrett32(r * e.mul, e.m, e.mu);
     v[i] = r;
   }
+  // staged tile: by TMA where u's rows allow it, else row by row
+  const int lane = threadIdx.x & 31;
+  const uint32_t buf = us.sbuf + (us.n & 1u) * 2048u;
   if (us.map != nullptr) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t buf = us.sbuf + (us.n & 1u) * 2048u;
     if (us.n >= 2) {                               // the buffer's previous store has read it
       if (lane == 0) tc::bulk_wait_read<1>();
       __syncwarp();
     }
+  } else {
+    // no TMA store may still read the buffer (a batch mixes both forms, and
+    // only TMA stores count as bulk groups: wait for all of them)
+    if (lane == 0) tc::bulk_wait_read<0>();
+    __syncwarp();
+  }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      tc::st_shared_v4(buf + (uint32_t)(lane * 64 + 16 * (q ^ ((lane >> 1) & 3))), v[8 * q] | (v[8 * q + 1] << 16),
-                       v[8 * q + 2] | (v[8 * q + 3] << 16), v[8 * q + 4] | (v[8 * q + 5] << 16),
-                       v[8 * q + 6] | (v[8 * q + 7] << 16));
+  for (int q = 0; q < 4; ++q)
+    tc::st_shared_v4(buf + (uint32_t)(lane * 64 + 16 * (q ^ ((lane >> 1) & 3))), v[8 * q] | (v[8 * q + 1] << 16),
+                     v[8 * q + 2] | (v[8 * q + 3] << 16), v[8 * q + 4] | (v[8 * q + 5] << 16),
+                     v[8 * q + 6] | (v[8 * q + 7] << 16));
+  ++us.n;
+  if (us.map != nullptr) {
     tc::fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) {
       tc::tma_store_3d(us.map, buf, col, e.row - lane, e.ell);   // rows >= M, columns >= N are not written
       tc::bulk_commit();
     }
-    ++us.n;
-    return;
-  }
-  if (e.row >= e.M) return;
-  if (e.vec_ok && col + 32 <= e.N) {
-    uint4* dst = reinterpret_cast<uint4*>(e.urow + col);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint4 w;
-      w.x = v[8 * q + 0] | (v[8 * q + 1] << 16);
-      w.y = v[8 * q + 2] | (v[8 * q + 3] << 16);
-      w.z = v[8 * q + 4] | (v[8 * q + 5] << 16);
-      w.w = v[8 * q + 6] | (v[8 * q + 7] << 16);
-      dst[q] = w;
-    }
   } else {
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (col + i < e.N) e.urow[col + i] = (uint16_t)v[i];
+    __syncwarp();
+    store_tile_rows(e.uell, buf, e.row - lane, col, e.M, e.N);
   }
 }
 
