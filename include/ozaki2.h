@@ -357,7 +357,8 @@ OZ2_API int ozaki2_zgemm(int64_t M, int64_t N, int64_t K, int p, const ozaki2_ma
 OZ2_API int ozaki2_gemm_batched(int count, const ozaki2_problem* probs, const ozaki2_opts* opts,
                         void* stream);
 
-/* Free the plans and workspaces cached by ozaki2_gemm / ozaki2_gemm_batched. */
+/* Free the plans and workspaces cached by ozaki2_gemm / ozaki2_gemm_batched /
+   ozaki2_zgemm, and the binary64 caches kept by ozaki2_cache_destroy. */
 OZ2_API int ozaki2_release_cache(void);
 
 /* Synchronise `stream` and read the plan's device status word:
@@ -398,6 +399,11 @@ OZ2_API int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, i
 OZ2_API int ozaki2_dgemm_bwd(ozaki2_cache cache, const double* dC, int64_t lddc, double* dA,
                      int64_t ldda, double* dB, int64_t lddb, void* stream);
 
+/* Give a cache back.  The library may keep its memory for the next
+   ozaki2_dgemm_fwd of the same shape and options on the same device (at most 32
+   caches and an eighth of the device's memory, none while less than a quarter of
+   it is free; freed by ozaki2_release_cache and before an allocation of the
+   library fails); the stream of that call waits for this cache's last run. */
 OZ2_API int ozaki2_cache_destroy(ozaki2_cache cache);
 
 /* ---------------------------------------------------------------------------

@@ -264,6 +264,16 @@ struct DevState {
   std::vector<Group> groups;
 };
 
+cudaError_t dev_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    release_retired_caches();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 static void free_launch_block(LaunchBlock& lb) {
   if (lb.copied) cudaEventSynchronize(lb.copied), cudaEventDestroy(lb.copied);
   if (lb.d_mem) cudaFree(lb.d_mem);
@@ -1262,7 +1272,7 @@ static int upload(ozaki2_plan_s* pl) {
   int rc = build_table_image(pl, sms, ti);
   if (rc) return rc;
   void* mem = nullptr;
-  if (injected_alloc_failure() || cudaMalloc(&mem, ti.b.img.size()) != cudaSuccess) return OZ2_ENOMEM;
+  if (injected_alloc_failure() || dev_malloc(&mem, ti.b.img.size()) != cudaSuccess) return OZ2_ENOMEM;
   if (cudaMemcpy(mem, ti.b.img.data(), ti.b.img.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaFree(mem);
     return OZ2_ECUDA;
@@ -1292,7 +1302,7 @@ static int alloc_launch_block(LaunchBlock& lb, int slots) {
   lb.tmap_off = probs_bytes;
   lb.bytes = probs_bytes + sizeof(CUtensorMap) * kMapsPerProblem * slots;
   int rc = OZ2_OK;
-  if (injected_alloc_failure() || cudaMalloc(&lb.d_mem, lb.bytes) != cudaSuccess) {
+  if (injected_alloc_failure() || dev_malloc(&lb.d_mem, lb.bytes) != cudaSuccess) {
     lb.d_mem = nullptr;
     rc = OZ2_ENOMEM;
   } else if (cudaMallocHost(&lb.h_stage, lb.bytes) != cudaSuccess) {
@@ -2135,7 +2145,7 @@ int cached_run(int count, const ozaki2_problem* probs, const ozaki2_opts* opts, 
     int rc = count == 1 ? ozaki2_plan_create(probs[0].M, probs[0].N, probs[0].K, probs[0].p, &o, &c.plan)
                         : ozaki2_plan_create_batched(count, probs, &o, &c.plan);
     if (rc) return rc;
-    if (cudaMalloc(&c.ws, c.plan->ws_bytes) != cudaSuccess) {
+    if (dev_malloc(&c.ws, c.plan->ws_bytes) != cudaSuccess) {
       ozaki2_plan_destroy(c.plan);
       return OZ2_ENOMEM;
     }
@@ -2173,7 +2183,7 @@ int ozaki2_zgemm(int64_t M, int64_t N, int64_t K, int p, const ozaki2_mat* Ar, c
       Cached c;
       int rc = ozaki2_plan_create_complex(M, N, K, p, &o, &c.plan);
       if (rc) return rc;
-      if (injected_alloc_failure() || cudaMalloc(&c.ws, c.plan->ws_bytes) != cudaSuccess) {
+      if (injected_alloc_failure() || dev_malloc(&c.ws, c.plan->ws_bytes) != cudaSuccess) {
         ozaki2_plan_destroy(c.plan);
         return OZ2_ENOMEM;
       }
@@ -2196,6 +2206,7 @@ int ozaki2_gemm_batched(int count, const ozaki2_problem* probs, const ozaki2_opt
 }
 
 int ozaki2_release_cache(void) {
+  release_retired_caches();
   std::lock_guard<std::mutex> lk(g_cache_mu);
   for (auto& kv : g_cache) {
     cudaFree(kv.second.ws);

@@ -14,6 +14,7 @@
 // modulus set for inner length max(M, N, K) so that the same planes serve all
 // three products.
 #include <algorithm>
+#include <list>
 #include <map>
 #include <mutex>
 #include <new>
@@ -131,8 +132,10 @@ struct ozaki2_cache_s {
   oz2::PlanFacts ff{}, fa{}, fb{};
   void* mem = nullptr;          // fwd workspace + A/B conversions
   void* mem_bwd = nullptr;      // backward workspaces + dC conversion
-  size_t bwd_bytes = 0;
+  size_t fwd_bytes = 0, bwd_bytes = 0;
   oz2::MpBuf a, b;
+  std::vector<int64_t> key;     // device, shape and options: what a later forward must match to take it over
+  cudaEvent_t done = nullptr;   // recorded after every run with this cache
 };
 
 namespace oz2 {
@@ -141,12 +144,87 @@ namespace {
 int cache_release(ozaki2_cache_s* c) {
   if (!c) return OZ2_EINVAL;
   if (c->mem || c->mem_bwd) cudaDeviceSynchronize();
+  if (c->done) cudaEventDestroy(c->done);
   if (c->fwd) ozaki2_plan_destroy(c->fwd);
   if (c->bwd_a) ozaki2_plan_destroy(c->bwd_a);
   if (c->bwd_b) ozaki2_plan_destroy(c->bwd_b);
   if (c->mem) cudaFree(c->mem);
   if (c->mem_bwd) cudaFree(c->mem_bwd);
   delete c;
+  return OZ2_OK;
+}
+
+// Retired caches (plans, workspaces and conversion buffers), kept for the next
+// forward of the same shape and options on the same device: making one takes
+// several device and pinned allocations, table uploads and a device-wide wait
+// when it is freed (a 4096^3 forward and backward: 8 of 20.1 ms).  Bounded: at
+// most kPoolCaches caches and an eighth of the device's memory, the oldest freed
+// first, and none kept while less than a quarter of the device's memory is
+// free; all freed by ozaki2_release_cache and when a library allocation fails.
+// A cache that is taken over makes the new stream wait for `done`, so its
+// buffers are not rewritten before their last readers, whatever their stream.
+constexpr size_t kPoolCaches = 32;
+std::mutex g_pool_mu;
+std::list<ozaki2_cache_s*> g_pool;   // oldest first
+
+size_t cache_bytes(const ozaki2_cache_s* c) { return c->fwd_bytes + c->bwd_bytes; }
+
+std::vector<int64_t> cache_key(int64_t M, int64_t N, int64_t K, const ozaki2_opts& o) {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  return {dev, M, N, K, o.guard_bits, o.t_bits, o.engine, o.k_chunk, o.grid, o.schedule, o.timing, o.crt_engine,
+          o.res_engine, o.plane_group, o.gemm_tile};
+}
+
+// Runs inside a stream capture are neither ordered by nor recorded in `done`
+// (an event outside the capture cannot be waited for); their cache is not kept.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
+// A retired cache of this key, or null; `s` then waits for its last run.
+ozaki2_cache_s* pool_take(const std::vector<int64_t>& key, cudaStream_t s) {
+  if (capturing(s)) return nullptr;
+  ozaki2_cache_s* c = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (auto it = g_pool.end(); it != g_pool.begin();) {       // the latest one: most likely still in L2
+      --it;
+      if ((*it)->key == key) {
+        c = *it;
+        g_pool.erase(it);
+        break;
+      }
+    }
+  }
+  if (c && cudaStreamWaitEvent(s, c->done, 0) != cudaSuccess) {
+    cache_release(c);
+    c = nullptr;
+  }
+  return c;
+}
+
+// Keep a cache that its owner has given back, or free it.
+int cache_retire(ozaki2_cache_s* c) {
+  if (!c) return OZ2_EINVAL;
+  size_t free_b = 0, total_b = 0;
+  int dev = -1;
+  if (!c->done || c->key.empty() || cudaGetDevice(&dev) != cudaSuccess || c->key[0] != dev ||
+      cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || free_b < total_b / 4 || cache_bytes(c) > total_b / 8)
+    return cache_release(c);
+  std::list<ozaki2_cache_s*> out;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    size_t held = cache_bytes(c);
+    for (const ozaki2_cache_s* q : g_pool) held += cache_bytes(q);
+    while (!g_pool.empty() && (held > total_b / 8 || g_pool.size() + 1 > kPoolCaches)) {
+      held -= cache_bytes(g_pool.front());
+      out.splice(out.end(), g_pool, g_pool.begin());
+    }
+    g_pool.push_back(c);
+  }
+  for (ozaki2_cache_s* q : out) cache_release(q);
   return OZ2_OK;
 }
 
@@ -165,7 +243,8 @@ int cache_build(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2
   if (!rc) rc = plan_query(c->fwd, &c->ff);
   if (rc) { cache_release(c); return rc; }
   const size_t bytes = al(c->ff.ws_bytes) + MpBuf::bytes((int)M, (int)K) + MpBuf::bytes((int)K, (int)N);
-  if (cudaMalloc(&c->mem, bytes) != cudaSuccess) { c->mem = nullptr; cache_release(c); return OZ2_ENOMEM; }
+  if (dev_malloc(&c->mem, bytes) != cudaSuccess) { c->mem = nullptr; cache_release(c); return OZ2_ENOMEM; }
+  c->fwd_bytes = bytes;
   auto* base = static_cast<uint8_t*>(c->mem);
   c->a.place(base + al(c->ff.ws_bytes), (int)M, (int)K);
   c->b.place(base + al(c->ff.ws_bytes) + MpBuf::bytes((int)M, (int)K), (int)K, (int)N);
@@ -198,8 +277,9 @@ int ensure_bwd(ozaki2_cache_s* c) {
   if (!rc) rc = plan_create_ex(c->K, c->N, c->M, 53, &c->opts, eb, &c->bwd_b);   // dB = A_hat^T * D2 (M x N)
   if (!rc) rc = plan_query(c->bwd_b, &c->fb);
   if (rc) return rc;
-  c->bwd_bytes = al(c->fa.ws_bytes) + al(c->fb.ws_bytes) + MpBuf::bytes((int)c->M, (int)c->N);
-  if (cudaMalloc(&c->mem_bwd, c->bwd_bytes) != cudaSuccess) { c->mem_bwd = nullptr; return OZ2_ENOMEM; }
+  const size_t bytes = al(c->fa.ws_bytes) + al(c->fb.ws_bytes) + MpBuf::bytes((int)c->M, (int)c->N);
+  if (dev_malloc(&c->mem_bwd, bytes) != cudaSuccess) { c->mem_bwd = nullptr; return OZ2_ENOMEM; }
+  c->bwd_bytes = bytes;
   return OZ2_OK;
 }
 
@@ -253,6 +333,16 @@ std::mutex g_mu;
 std::map<std::vector<int64_t>, ozaki2_cache_s*> g_nocache;   // forwards without a cache handle
 
 }  // namespace
+
+void release_retired_caches() {
+  std::list<ozaki2_cache_s*> out;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    out.swap(g_pool);
+  }
+  for (ozaki2_cache_s* c : out) cache_release(c);
+}
+
 }  // namespace oz2
 
 using namespace oz2;
@@ -264,19 +354,34 @@ int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t l
                      void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   try {
-    if (cache_out) {
-      *cache_out = nullptr;
-      ozaki2_cache_s* c = nullptr;
-      int rc = cache_build(M, N, K, opts, &c);
-      if (rc) return rc;
-      rc = run_fwd(c, A, lda, B, ldb, Cd, ldc, s);
-      if (rc) { cache_release(c); return rc; }
-      *cache_out = c;
-      return OZ2_OK;
-    }
     ozaki2_opts o;
     if (opts) o = *opts;
     else ozaki2_opts_default(&o);
+    if (cache_out) {
+      *cache_out = nullptr;
+      if (!A || !B || !Cd || lda < K || ldb < N || ldc < N) {      // refused before a retired cache is taken
+        ozaki2_cache_s* c = nullptr;
+        const int rc = cache_build(M, N, K, &o, &c);
+        if (rc) return rc;
+        cache_release(c);
+        return OZ2_EINVAL;
+      }
+      auto key = cache_key(M, N, K, o);
+      ozaki2_cache_s* c = pool_take(key, s);
+      if (!c) {
+        const int rc = cache_build(M, N, K, &o, &c);
+        if (rc) return rc;
+      }
+      const int rc = run_fwd(c, A, lda, B, ldb, Cd, ldc, s);
+      if (rc) { cache_release(c); return rc; }
+      c->key.clear();                                // kept later only if its runs are recorded
+      if (!capturing(s)) {
+        if (!c->done && cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess) c->done = nullptr;
+        if (c->done && cudaEventRecord(c->done, s) == cudaSuccess) c->key = std::move(key);
+      }
+      *cache_out = c;
+      return OZ2_OK;
+    }
     int dev = -1;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(g_mu);
@@ -299,12 +404,17 @@ int ozaki2_dgemm_bwd(ozaki2_cache cache, const double* dC, int64_t lddc, double*
                      int64_t lddb, void* stream) {
   if (!cache) return OZ2_EINVAL;
   try {
-    return run_bwd(cache, dC, lddc, dA, ldda, dB, lddb, static_cast<cudaStream_t>(stream));
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // ordered after the cache's earlier runs, and recorded for the later ones
+    const bool ordered = !cache->key.empty() && !capturing(s) && cudaStreamWaitEvent(s, cache->done, 0) == cudaSuccess;
+    const int rc = run_bwd(cache, dC, lddc, dA, ldda, dB, lddb, s);
+    if (!ordered || cudaEventRecord(cache->done, s) != cudaSuccess) cache->key.clear();
+    return rc;
   } catch (const std::bad_alloc&) {
     return OZ2_ENOMEM;
   }
 }
 
-int ozaki2_cache_destroy(ozaki2_cache cache) { return cache_release(cache); }
+int ozaki2_cache_destroy(ozaki2_cache cache) { return cache_retire(cache); }
 
 }  // extern "C"

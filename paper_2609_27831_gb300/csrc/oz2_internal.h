@@ -203,6 +203,11 @@ cudaError_t launch_residues_mm(const DevTables& t, const int32_t* tiles, int nti
 void residue_mm_geometry(int kpad, int npad, int* cw, int* nabuf);
 int residue_mm_smem_bytes(int cw_max, int lmax, int tcols, int* stages);
 
+// cudaMalloc that frees the binary64 mode's retired caches and tries once more
+// before it reports a failure.
+cudaError_t dev_malloc(void** p, size_t bytes);
+void release_retired_caches();
+
 // Internal plan variants used by the binary64 mode.
 struct PlanExtra {
   int64_t inner = 0;     // choose moduli for inner length max(K, inner)
