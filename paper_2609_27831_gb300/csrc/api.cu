@@ -159,6 +159,7 @@ struct CrtHost {
   std::vector<uint32_t> words;   // pool layout (see CrtView), DS-padded
   // tensor-core CRT table B [npad][kpad] (bf16 bits): B[j][2l] = M_l[j],
   // B[j][2l+1] = M_l[j-1], M_l[j] the 7-bit pieces of M_l
+  int mode = 0;                               // crt_mode that the table serves (2: with the quotient columns)
   int kpad = 0, npad = 0, np = 0, rows = 0;   // rows: table rows allocated (>= npad)
   std::vector<uint16_t> tc_table;
 };
@@ -182,7 +183,8 @@ struct ProbHost {
   bool skip_a, skip_b;         // planes of that side are written by the caller
   int crt_mode;                // 0: CUDA-core CRT class crt_cls; 1: tensor-core CRT (class crt_cls);
                                // 2: tensor-core sums to R digits, then the finish
-  int crt_kpad, crt_npad, crt_np, crt_nchunk, crt_cw, crt_ngrp, crt_nslot, crt_nvbuf;
+  int crt_kpad, crt_npad, crt_np, crt_ngrp;
+  int crt_qgrp;                // crt_mode 2: groups that the workspace has room for
   int crt_gskip = 0;            // crt_mode 2, long finish: lowest group of Y columns formed
   size_t off_q, off_sig;       // crt_mode 2: group sums [ngrp][9][upitch] uint32, quotient estimates [upitch] uint32
   int res_mode, res_kpad, res_npad, res_key;   // tensor-core residues (table index res_key)
@@ -245,7 +247,7 @@ struct DevState {
   std::vector<int> crt_off;    // per problem, uint32 offset in the pool
   ListRef tct[9];               // tensor-core CRT tile lists (smem = kpad_max, lmax = L max)
   int tct_npad[9] = {0};
-  std::vector<ListRef> cmt;     // tensor-core CRT sum tiles, one list per TMEM layout (smem = chunk width)
+  ListRef cmt;                  // tensor-core CRT sums: runs of tiles (smem = most formed columns, lmax = most K blocks)
   ListRef finl;                 // finish blocks of long accumulators (smem = D max, lmax = output limbs max)
   ListRef fsh[9];               // finish blocks of one-lane classes after the tensor-core sums
   std::vector<ListRef> rmt;     // warp-specialised tensor-core residue tiles, one list per TMEM layout (smem = cw)
@@ -397,6 +399,18 @@ static int res_table_key(ozaki2_plan_s* pl, int l0, int L, int L1, int nb, int k
   return (int)pl->rtabs.size() - 1;
 }
 
+// Groups of 32 column sums that the workspace holds for `cols` formed columns:
+// whole chunks of the columns that two (or one, for chunks of 128 and more) of
+// the accumulator slots beside V take, kpad / 2 of the 512 TMEM columns.  The sums
+// kernel no longer runs in such chunks and forms cols / 32 groups; the workspace
+// of a shape stays what it was.
+static int crt_workspace_groups(int kpad, int npad, int cols) {
+  int cw = std::min(256, ((512 - kpad / 2) / 2) & ~31);
+  if (cw < 128 && cw < npad) cw = std::min(256, (512 - kpad / 2) & ~31);
+  cw = std::min(cw, npad);
+  return (cols + cw - 1) / cw * cw / 32;
+}
+
 // One problem of a plan.  `po` (batched plans) supplies this problem's own
 // guard bits, t, K chunk and residue and CRT engines; the plan's options
 // otherwise.
@@ -492,24 +506,16 @@ static int build_problem(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int
     // (measured at 1024^3: 0.238 vs 0.248 ms at 21 digits, 0.27 vs 0.33 at 25,
     // 0.42 vs 0.67 at 33; 0.21 vs 0.18 at 17), the one-lane CUDA-core CRT below
     const bool want_mm = o.crt_engine == 2 || (o.crt_engine == 0 && h.D32 > 20);
-    // sums of any length: fp32 column sums exact for 2L 127^2 < 2^24, and V
-    // for 128 outputs (kpad bf16 each) plus the rings must fit in shared memory
-    // (the u copies are boxes of 32 moduli x 128 outputs: at least that many;
-    // V takes kpad / 2 of the 512 TMEM columns, two accumulator slots the rest)
+    // sums of any length: fp32 column sums exact for 2L 127^2 < 2^24 (the u
+    // copies are boxes of 32 moduli x 128 outputs: at least that many)
     const bool mm_ok = want_mm && 2 * L * 127 * 127 < (1 << 24) && L >= 32 && M * N >= 128 &&
                        kpad / 2 + 2 * 32 <= 512;
     h.crt_mode = tc_ok ? 1 : (mm_ok ? 2 : 0);
     h.crt_kpad = kpad;
     h.crt_npad = h.crt_mode == 2 ? npad_mm : npad;
     h.crt_np = np;
-    h.crt_nslot = 2;
-    h.crt_cw = mm_ok ? crt_mm_chunk(kpad, npad_mm, &h.crt_nslot) : 0;
-    h.crt_nchunk = mm_ok ? (npad_mm + h.crt_cw - 1) / h.crt_cw : 0;
-    // a second V buffer where it fits beside the accumulator slots: the
-    // next tile's V is built while this tile's chunks are read out
-    h.crt_nvbuf = (mm_ok && kpad + h.crt_nslot * h.crt_cw <= 512) ? 2 : 1;
-    h.crt_ngrp = mm_ok ? h.crt_nchunk * h.crt_cw / 32 : 0;
-    const int rows = h.crt_mode == 2 ? h.crt_cw * h.crt_nchunk : npad;
+    h.crt_ngrp = mm_ok ? npad_mm / 32 : 0;
+    const int rows = h.crt_mode == 2 ? npad_mm : npad;
     // The finish of long accumulators reads the group sums from group g0 - 1
     // on in its fast form (g0: the group whose lowest digit lies just below
     // its window of the 2 nl + 4 highest digits), and takes an output's full
@@ -521,18 +527,21 @@ static int build_problem(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int
       const int g0 = wbase > 7 ? (wbase - 1) / 7 : 0;
       if (g0 >= 2) {
         h.crt_gskip = g0 - 1;
-        h.crt_nchunk = (npad_mm - 32 * h.crt_gskip + h.crt_cw - 1) / h.crt_cw;
-        h.crt_ngrp = h.crt_nchunk * h.crt_cw / 32;
+        h.crt_ngrp -= h.crt_gskip;
       }
     }
+    h.crt_qgrp = mm_ok ? crt_workspace_groups(kpad, npad_mm, 32 * h.crt_ngrp) : 0;
+    if (h.crt_mode == 2 && !crt_mm_fits(32 * h.crt_ngrp)) return OZ2_EINTERNAL;
     CrtHost* cp = &c;
-    if (h.crt_mode != 0 && !c.tc_table.empty() && (c.rows != rows || c.npad != h.crt_npad)) {
+    if (h.crt_mode != 0 && !c.tc_table.empty() && (c.mode != h.crt_mode || c.rows != rows || c.npad != h.crt_npad)) {
       // another problem of this modulus set runs the other tensor-core CRT
       // form: a table of this form exists already, or this problem gets a copy
       // of the digit tables with its own
       int other = -1;
       for (size_t i = 0; i < pl->crts.size(); ++i)
-        if (pl->crts[i].L == L && pl->crts[i].rows == rows && pl->crts[i].npad == h.crt_npad) other = (int)i;
+        if (pl->crts[i].L == L && pl->crts[i].mode == h.crt_mode && pl->crts[i].rows == rows &&
+            pl->crts[i].npad == h.crt_npad)
+          other = (int)i;
       if (other < 0) {
         CrtHost cc;
         cc.L = c.L; cc.D32 = c.D32; cc.DS = c.DS; cc.cls = c.cls; cc.P = c.P; cc.words = c.words;
@@ -545,7 +554,7 @@ static int build_problem(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int
     CrtHost& c2 = *cp;
     if (h.crt_mode != 0 && c2.tc_table.empty()) {
       CrtHost& c = c2;
-      c.kpad = kpad; c.npad = h.crt_npad; c.np = np; c.rows = rows;
+      c.mode = h.crt_mode; c.kpad = kpad; c.npad = h.crt_npad; c.np = np; c.rows = rows;
       c.tc_table.assign((size_t)rows * kpad, 0);
       const auto& mlist = modulus_list();
       auto bf = [](uint32_t x) -> uint16_t {   // exact for x <= 256
@@ -738,7 +747,7 @@ static void layout_workspace(ozaki2_plan_s* pl) {
     h.off_q = h.off_sig = off;
     if (h.crt_mode == 2) {
       const size_t up = align_up((size_t)(h.M * h.N), 8);
-      off += align_up(4 * (size_t)h.crt_ngrp * 9 * up, 256);
+      off += align_up(4 * (size_t)h.crt_qgrp * 9 * up, 256);
       h.off_sig = off;
       off += align_up(4 * up, 256);               // quotient estimates
     }
@@ -824,10 +833,11 @@ struct TableImage {
   size_t o_tct[9] = {0};
   int n_tct[9] = {0}, tct_kpad[9] = {0}, tct_npad[9] = {0}, tct_l[9] = {0};
   std::vector<size_t> o_tctab;
-  // tensor-core CRT sum tiles and warp-specialised tensor-core residue
+  // tensor-core CRT sums: runs of tiles; warp-specialised tensor-core residue
   // tiles: one launch per TMEM layout, {first tile, tiles, chunk width}
   size_t o_cmt = 0, o_finl = 0;
-  std::vector<std::array<int, 3>> cmt_seg, rmt_seg;
+  int n_cmt = 0, cmt_cols = 0, cmt_kb = 0;
+  std::vector<std::array<int, 3>> rmt_seg;
   size_t o_fsh[9] = {0};            // short finish blocks per one-lane class (after the tensor-core sums)
   int n_fsh[9] = {0};
   int n_finl = 0, finl_dmax = 0, finl_nlmax = 0;
@@ -1014,7 +1024,8 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
   std::vector<int4> rtt, finl;
   // tiles of the warp-specialised kernels grouped by TMEM layout (tiles of
   // one launch share the column map of their buffers and slots)
-  std::map<std::array<int, 3>, std::vector<int4>> cmt_by, rmt_by;
+  std::map<std::array<int, 3>, std::vector<int4>> rmt_by;
+  std::vector<int4> cmt;
   for (int pi = 0; pi < count; ++pi) {
     const ProbHost& h = pl->probs[pi];
     const bool own_planes = !h.sum_of;             // planes made by the scan and residue kernels
@@ -1070,8 +1081,11 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
       // from the group below the window on)
       const int64_t nt = (h.M * h.N + 127) / 128;
       if (nt > INT_MAX) return OZ2_ERANGE;
-      std::vector<int4>& cl = cmt_by[{h.crt_kpad, h.crt_cw, h.crt_nslot}];
-      for (int64_t tt = 0; tt < nt; ++tt) cl.push_back(make_int4(pi, (int)tt, 0, 0));
+      if (nt > INT_MAX - ti.n_cmt) return OZ2_ERANGE;
+      cmt.push_back(make_int4(pi, ti.n_cmt, ti.n_cmt + (int)nt, 0));
+      ti.n_cmt += (int)nt;
+      ti.cmt_cols = std::max(ti.cmt_cols, 32 * h.crt_ngrp);
+      ti.cmt_kb = std::max(ti.cmt_kb, h.crt_kpad / 64);
       if (h.crt_cls <= 4) {
         for (int64_t bb = 0; bb < nt; ++bb) fsh[h.crt_cls].push_back(make_int4(pi, (int)bb, 0, 0));
       } else {
@@ -1135,16 +1149,12 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
       return OZ2_EINTERNAL;
     if (h.crt_mode == 0 && ti.crt_l[h.crt_cls] < h.L) return OZ2_EINTERNAL;
     if (h.crt_mode == 1 && (ti.tct_l[h.crt_cls] < h.L || ti.tct_kpad[h.crt_cls] < h.crt_kpad)) return OZ2_EINTERNAL;
-    if (h.crt_mode == 2 && (h.crt_cw % 32 != 0 || h.crt_nvbuf * (h.crt_kpad / 2) + h.crt_nslot * h.crt_cw > 512 ||
+    if (h.crt_mode == 2 && (h.crt_ngrp > h.crt_qgrp ||
                             (h.crt_cls > 4 && (ti.finl_dmax < h.D32 || ti.finl_nlmax < h.nl))))
       return OZ2_EINTERNAL;
   }
-  std::vector<int4> cmt, rmt;
-  for (const auto& kv : cmt_by) {
-    if (crt_mm_smem_bytes(kv.first[1], pl->lmax, nullptr) < 0) return OZ2_EINTERNAL;
-    ti.cmt_seg.push_back({(int)cmt.size(), (int)kv.second.size(), kv.first[1]});
-    cmt.insert(cmt.end(), kv.second.begin(), kv.second.end());
-  }
+  std::vector<int4> rmt;
+  if (ti.n_cmt > 0 && !crt_mm_fits(ti.cmt_cols)) return OZ2_EINTERNAL;
   ti.na_rmt.clear();
   for (const auto& kv : rmt_by) {
     if (residue_mm_smem_bytes(kv.first[1], pl->lmax, 512, nullptr) < 0) return OZ2_EINTERNAL;
@@ -1213,9 +1223,7 @@ static void install_table_image(ozaki2_plan_s* pl, const TableImage& ti, uint8_t
     d.tct[i] = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_tct[i]), ti.n_tct[i], ti.tct_kpad[i], ti.tct_l[i]};
     d.tct_npad[i] = ti.tct_npad[i];
   }
-  d.cmt.clear();
-  for (const auto& sg : ti.cmt_seg)
-    d.cmt.push_back(ListRef{reinterpret_cast<const int32_t*>(base + ti.o_cmt) + 4 * sg[0], sg[1], sg[2], 0});
+  d.cmt = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_cmt), ti.n_cmt, ti.cmt_cols, ti.cmt_kb};
   d.finl = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_finl), ti.n_finl, ti.finl_dmax, ti.finl_nlmax};
   for (int c = 0; c < 9; ++c) d.fsh[c] = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_fsh[c]), ti.n_fsh[c], 0, 0};
   d.rtt = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_rtt), ti.n_rtt, ti.rtt_kpad, ti.rtt_l, ti.na_rtt};
@@ -1411,14 +1419,10 @@ static int build_image(ozaki2_plan_s* pl, const ozaki2_problem* probs, uint8_t* 
     P.crt_kpad = h.crt_kpad;
     P.crt_npad = h.crt_npad;
     P.crt_np = h.crt_np;
-    P.crt_nchunk = h.crt_nchunk;
-    P.crt_cw = h.crt_cw;
     P.crt_q = h.crt_mode == 2 ? reinterpret_cast<uint32_t*>(ws + h.off_q) : nullptr;
     P.crt_alpha = h.crt_mode == 2 ? reinterpret_cast<uint32_t*>(ws + h.off_sig) : nullptr;
     P.crt_ngrp = h.crt_ngrp;
     P.crt_gskip = h.crt_gskip;
-    P.crt_nslot = h.crt_nslot;
-    P.crt_nvbuf = h.crt_nvbuf;
     int rc = encode_planes(&tm[2 * i], P.pa, h.K, h.M, h.Kp, h.G, kBM);
     if (rc) return rc;
     rc = encode_planes(&tm[2 * i + 1], P.pb, h.K, h.N, h.Kp, h.G, pl->tile2 ? kBN / 2 : kBN);
@@ -1426,12 +1430,11 @@ static int build_image(ozaki2_plan_s* pl, const ozaki2_problem* probs, uint8_t* 
     rc = encode_u_store(&tm[5 * count + i], P.u, h.N, h.M, h.L, P.upitch, &P.u_map);
     if (rc) return rc;
     if (h.crt_mode != 0) {
-      // mode 1: the whole table in K blocks; mode 2: K block x cw columns of
-      // a table padded to whole chunks
+      // mode 1: the whole table in K blocks; mode 2: K block x 32 columns
       const int rows = pl->crts[h.crt_key].rows;
       const cuuint64_t dims[2] = {(cuuint64_t)h.crt_kpad, (cuuint64_t)rows};
       const cuuint64_t strides[1] = {(cuuint64_t)h.crt_kpad * 2};
-      const cuuint32_t box[2] = {64u, (cuuint32_t)(h.crt_mode == 1 ? h.crt_npad : h.crt_cw)};
+      const cuuint32_t box[2] = {64u, (cuuint32_t)(h.crt_mode == 1 ? h.crt_npad : 32)};
       const cuuint32_t es[2] = {1u, 1u};
       if (get_encode()(&tm[2 * count + i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pl->dev.crt_tab[i], dims, strides,
                        box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1591,17 +1594,7 @@ static int enqueue(ozaki2_plan_s* pl, LaunchBlock& lb, uint8_t* ws, cudaStream_t
     OZ2_CU(launch_combine_complex(tab, (int64_t)h.L * (int64_t)(align_up((size_t)(h.M * h.N), 8) / 8), s));
   }
   if (timing) OZ2_CU(cudaEventRecord(pl->ev[3], s));
-  {
-    // the CRT table stays resident in the sums kernel when one problem uses it
-    int n2 = 0, blocks_one = 0;
-    for (const ProbHost& h : pl->probs)
-      if (h.crt_mode == 2 && !h.no_crt) {
-        ++n2;
-        blocks_one = (h.crt_kpad / 64) * h.crt_nchunk;
-      }
-    for (const ListRef& r : d.cmt)
-      OZ2_CU(launch_crt_mm(tab, r.ptr, r.n, r.smem, d.sms, n2 == 1 ? blocks_one : 0, s));
-  }
+  if (d.cmt.n) OZ2_CU(launch_crt_mm(tab, d.cmt.ptr, d.cmt.n, d.cmt.smem, d.cmt.lmax, d.sms, s));
   if (timing) OZ2_CU(cudaEventRecord(pl->ev[5], s));
   for (int c = 0; c < 9; ++c)
     if (d.fsh[c].n) OZ2_CU(launch_crt_fin_short(tab, c, d.fsh[c].ptr, d.fsh[c].n, s));
@@ -1913,7 +1906,7 @@ int ozaki2_plan_launches(ozaki2_plan pl, int* n) {
   else if (pl->opts.engine == OZ2_ENGINE_SIMT || pl->opts.engine == OZ2_ENGINE_S8) c += res + 1;
   else if (pl->opts.schedule == OZ2_SCHED_GROUPED) c += res + 1;
   else c += res + (int)d.plain.size();
-  c += (int)d.cmt.size();
+  c += d.cmt.n ? 1 : 0;
   c += d.finl.n ? 1 : 0;
   for (int i = 0; i < 9; ++i) c += d.fsh[i].n ? 1 : 0;
   for (int i = 0; i < kCrtClassCount; ++i) c += d.crt[i].n ? 1 : 0;

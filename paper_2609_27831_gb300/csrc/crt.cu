@@ -1201,13 +1201,27 @@ __global__ void __launch_bounds__(kFinThreads, (ND <= 24 ? 6 : 1)) k_crt_fin_sho
 // an exact integer below 2L 127^2 < 2^24 for L <= 520.  The plane GEMM
 // already stored v_l = u_l M_l^{-1} mod m_l in place of u_l.
 //
-// Per tile of 128 consecutive outputs, V lives in tensor memory: TMEM lane r
-// holds output r's row, column l the bf16 pair (v0_l, v1_l).  The columns of
-// Y run in chunks of cw (a multiple of 32) through two TMEM accumulator slots
-// after V (kpad / 2 + 2 cw <= 512), or through one slot when two would make
-// the MMAs narrower than 128 columns; the B blocks (64 k x cw columns) stream
-// through a shared-memory ring.  32 consecutive pieces span exactly 7 words,
-// so group g of 32 columns is the integer
+// Per tile of 128 consecutive outputs every formed column of Y is accumulated in
+// one pass over K: K block q (64 k) is the 32 moduli 32 q .. 32 q + 31, whose v
+// values arrive as one TMA copy, are split into bf16 halves by the builders and
+// written as a 128 x 64 operand block; two MMAs per K step take the first 256
+// columns and the rest.  Tensor memory holds accumulators only:
+//   up to 256 columns (launch-wide): two slots of 256, tiles in turn
+//   more (at most 384): one slot of 256 for the first chunk and two for the
+//   rest; the next tile's MMAs wait for the first chunk to be read out.
+// What bounds it: the chain of V block, MMAs and read-out per tile, and beside it
+// the table's 0.5 MB per tile from L2 where it does not stay in the ring; the
+// sums' 9 words per group are 0.45 GB at 1024^3 p = 2048.  The MMA issuer is a
+// converged warp with one elected lane: issued from a single-lane branch, whose
+// descriptors are not warp-uniform, each MMA took 100 to 140 cycles whatever its
+// N (0.56 ms at 1024^3 p = 2048 for the 0.48 below).  An earlier form kept V in
+// tensor memory, 352 columns at p = 2048, and ran the columns in chunks of 160
+// through the one slot left, V build, MMAs and epilogues in turn.  Earlier form
+// and now, ms: 1024^3 p = 256 0.130 and 0.102, p = 1024 0.447 and 0.231, p = 2048
+// 0.98 and 0.48; 4096^3 p = 2048 16.4 and 7.9.  (12 epilogue warps: 1 to 2 % more.)
+//
+// 32 consecutive pieces span exactly 7 words, so group g of 32 columns is the
+// integer
 //   Q_g = sum_{q < 32} Y_{32 g + q} 2^(7 q),   S = sum_g Q_g 2^(224 g),
 // with piece q in word 7 q / 32 at shift 7 q mod 32 (both constants); each
 // Q_g is written on its own as 9 words (7 carried word sums and the carry),
@@ -1215,43 +1229,60 @@ __global__ void __launch_bounds__(kFinThreads, (ND <= 24 ? 6 : 1)) k_crt_fin_sho
 // crt_gskip > 0 (the long finish, whose fast form reads no lower group) the
 // columns start at 32 crt_gskip: the groups below are not formed, and stored
 // group i is group crt_gskip + i.
-//   warp 0      TMA producer of the B blocks, in (chunk, K block) order
-//   warp 1      MMA issuer: chunks into the slots in turn (one slot: always
-//               slot 0); commits per ring stage, per chunk and per tile
-//   warp 2      TMA producer of the tile's v values, 32 moduli x 128 outputs
-//               per copy, into a four-slot ring
-//   warps 3-18  four threads per output (its TMEM lane), groups h = 0..3:
-//               group h writes the V columns of the copies c = h mod 4 (in
-//               pieces of 8 columns); then the tile's 32-column groups in
-//               turn.  The last group's columns 27..31 are the sums of the
-//               pieces of floor(2^28 / m_l): the quotient estimate
-//               alpha~ = floor(sum_l v_l floor(2^28 / m_l) / 2^28), in
-//               {alpha - 1, alpha}, written per output for the finish.
-// A warp rewrites its V columns only after the commit that follows the
-// previous tile's last MMA, and the next tile's MMAs wait for every warp's V
-// columns (tcgen05.st waited and fenced), so V is never read and written at
-// once; an accumulator slot is reused only after every worker has read it.
-// Tile list entry: {problem, tile, 0, 0}.
+//   warp 0       TMA producer of the table: stages of 64 k x the problem's
+//                columns, in boxes of 32 columns; a problem whose table fits in
+//                the ring keeps it there from its first tile to its last here
+//   warp 1       MMA issuer: commits per V block, per table stage, per tile
+//   warp 2       TMA producer of the v values, 32 moduli x 128 outputs per copy
+//   warps 3-10   builders: two threads per output row, 16 moduli of a block each
+//   warps 11-26  epilogue, four per TMEM lane quadrant: the tile's 32-column
+//                groups in turn.  The last group's columns 27..31 are the sums
+//                of the pieces of floor(2^28 / m_l): the quotient estimate
+//                alpha~ = floor(sum_l v_l floor(2^28 / m_l) / 2^28), in
+//                {alpha - 1, alpha}, written per output for the finish.
+// Runs of tiles: {problem, first tile, end, 0}.
 // ---------------------------------------------------------------------------
-constexpr int kCmWorkers = 512;
-constexpr int kCmThreads = 96 + kCmWorkers;
-constexpr int kCmMaxStages = 24;
+constexpr int kCmBuildWarps = 8, kCmEpiWarps = 16;
+constexpr int kCmThreads = 32 * (3 + kCmBuildWarps + kCmEpiWarps);
+constexpr int kCmMaxStages = 12;
 constexpr int kCmUMods = 32;                         // moduli per v copy
-constexpr int kCmUSlots = 4;
+constexpr int kCmMinUSlots = 2, kCmMaxUSlots = 8;
 constexpr uint32_t kCmUBytes = kCmUMods * 128 * 2;   // [32][128] uint16
+constexpr int kCmVSlots = 4;
+constexpr uint32_t kCmVBytes = 128 * 128;            // 128 outputs x 64 k bf16
 constexpr int kCmMinSmem = 116 * 1024;               // one CTA per SM: it holds all 512 TMEM columns
+constexpr int kCmWide = 256;                         // columns of the first chunk
+constexpr int kCmCols = kCmWide + (512 - kCmWide) / 2;   // most columns: two slots of the rest
 
 struct CmLayout {
-  uint32_t ring_off, u_off, mu_off, bar_off, total;
-  __host__ __device__ CmLayout(uint32_t stage_bytes, int stages, int lmax) {
-    ring_off = 0;
-    u_off = (uint32_t)stages * stage_bytes;
-    mu_off = u_off + kCmUSlots * kCmUBytes;                 // floor(2^32 / m_l) [lmax]
-    bar_off = mu_off + (((uint32_t)lmax * 4 + 15u) & ~15u);
-    // barriers: full, empty [kCmMaxStages], u_full, u_free [kCmUSlots], acc_full, acc_free [2],
-    // v_full, v_free [2], drain; then the abort flag and the TMEM slot
-    total = 1024 + bar_off + (2 * kCmMaxStages + 2 * kCmUSlots + 9) * 8 + 16;
+  uint32_t v_off, u_off, bar_off, total;
+  __host__ __device__ CmLayout(uint32_t stage_bytes, int stages, int uslots) {
+    v_off = (uint32_t)stages * stage_bytes;
+    u_off = v_off + kCmVSlots * kCmVBytes;
+    bar_off = u_off + (uint32_t)uslots * kCmUBytes;
+    // barriers: full, empty [kCmMaxStages], u_full, u_free [kCmMaxUSlots], v_full, v_free [kCmVSlots],
+    // acc_full, a_free, b_free [2], drain; then the abort flag and the TMEM slot
+    total = 1024 + bar_off + (2 * kCmMaxStages + 2 * kCmMaxUSlots + 2 * kCmVSlots + 7) * 8 + 16;
     if (total < (uint32_t)kCmMinSmem) total = kCmMinSmem;
+  }
+};
+
+// A run of a problem's tiles in the launch; every role walks the runs on its own.
+struct CmWalk {
+  const int4* seg;
+  int prob, first, end;
+  __device__ CmWalk(const int4* s) : seg(s - 1), prob(-1), first(0), end(0) {}
+  __device__ bool seek(int i) {                      // to the run of tile i; true if it is another one
+    bool moved = false;
+    while (i >= end) {
+      ++seg;
+      const int4 a = __ldg(seg);
+      prob = a.x;
+      first = a.y;
+      end = a.z;
+      moved = true;
+    }
+    return moved;
   }
 };
 
@@ -1260,7 +1291,6 @@ __device__ __forceinline__ uint32_t f2u_exact24(uint32_t bits) {
   const float f = __uint_as_float(bits);
   return f >= 8388608.0f ? bits - 0x4A800000u : __float_as_uint(f + 8388608.0f) - 0x4B000000u;
 }
-
 
 // {bf16(v mod 128), bf16(floor(v / 128))} for v < 2^14 (low half, high half):
 // 2^23 + x has x in its low mantissa bits; both halves are exact in bf16
@@ -1300,47 +1330,51 @@ __device__ __forceinline__ void crt_group_small(const uint32_t* y, uint64_t (&ac
   for (int w = 0; w < 7; ++w) acc[w] -= crt_group_bias<NQ>(w);
 }
 
-template <bool resident>
 __global__ void __launch_bounds__(kCmThreads, 1)
-    k_crt_mm(const __grid_constant__ DevTables T, const int4* __restrict__ tiles, int ntiles, uint32_t stage_bytes,
-             int stages) {
+    k_crt_mm(const __grid_constant__ DevTables T, const int4* __restrict__ segs, int ntiles, uint32_t stage_bytes,
+             int stages, int uslots, int cmax) {
   using namespace tc;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* sm = smem_raw + (base - raw);
-  const CmLayout lay(stage_bytes, stages, T.lmax);
-  const uint32_t sRing = base + lay.ring_off;                 // B ring [stages][cw cols][128 B]
-  const uint32_t sU = base + lay.u_off;                       // v ring [kCmUSlots][32][128] uint16
+  const CmLayout lay(stage_bytes, stages, uslots);
+  const uint32_t sRing = base;                                // table ring [stages][columns][128 B]
+  const uint32_t sV = base + lay.v_off;                       // V ring [kCmVSlots][128][128 B]
+  const uint32_t sU = base + lay.u_off;                       // v ring [uslots][32][128] uint16
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + lay.bar_off);
   uint64_t* full = bars;                                      // [kCmMaxStages]
-  uint64_t* empty = bars + kCmMaxStages;                      // [kCmMaxStages]
-  uint64_t* u_full = bars + 2 * kCmMaxStages;                 // [kCmUSlots]
-  uint64_t* u_free = u_full + kCmUSlots;                      // [kCmUSlots] (128 arrivals: one half)
-  uint64_t* acc_full = u_free + kCmUSlots;                    // [2] chunk in slot done
-  uint64_t* acc_free = acc_full + 2;                          // [2] slot read out (256 arrivals)
-  uint64_t* v_full = acc_free + 2;                            // [2] V buffer written (every worker)
-  uint64_t* v_free = v_full + 2;                              // [2] MMAs reading the buffer done
-  uint64_t* drain = v_full + 4;                               // abort drain of the MMA pipe
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(v_full + 5);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(v_full + 5) + 1;
+  uint64_t* empty = full + kCmMaxStages;                      // [kCmMaxStages]
+  uint64_t* u_full = empty + kCmMaxStages;                    // [kCmMaxUSlots]
+  uint64_t* u_free = u_full + kCmMaxUSlots;                   // [kCmMaxUSlots] (one arrival per builder warp)
+  uint64_t* v_full = u_free + kCmMaxUSlots;                   // [kCmVSlots] (one arrival per builder warp)
+  uint64_t* v_free = v_full + kCmVSlots;                      // [kCmVSlots] MMAs reading the block done
+  uint64_t* acc_full = v_free + kCmVSlots;                    // [2] tile t's columns complete: barrier t & 1
+  uint64_t* a_free = acc_full + 2;                            // [2] tile t's first chunk read (one arrival per warp)
+  uint64_t* b_free = a_free + 2;                              // [2] ... and the rest
+  uint64_t* drain = b_free + 2;                               // abort drain of the MMA pipe
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(drain + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1) + 1;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kCmMaxStages; ++i) {
       mbar_init(full + i, 1);
       mbar_init(empty + i, 1);
     }
-    for (int i = 0; i < kCmUSlots; ++i) {
+    for (int i = 0; i < kCmMaxUSlots; ++i) {
       mbar_init(u_full + i, 1);
-      mbar_init(u_free + i, 128);
+      mbar_init(u_free + i, kCmBuildWarps);
     }
-    for (int i = 0; i < 2; ++i) mbar_init(acc_full + i, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(v_full + i, kCmWorkers);
+    for (int i = 0; i < kCmVSlots; ++i) {
+      mbar_init(v_full + i, kCmBuildWarps);
       mbar_init(v_free + i, 1);
     }
-    for (int i = 0; i < 2; ++i) mbar_init(acc_free + i, kCmWorkers);   // every worker reads every chunk
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(acc_full + i, 1);
+      mbar_init(a_free + i, kCmEpiWarps);
+      mbar_init(b_free + i, kCmEpiWarps);
+    }
     mbar_init(drain, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1354,30 +1388,39 @@ __global__ void __launch_bounds__(kCmThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // slots of the first chunk and of the rest, and where they start (launch-wide)
+  const int rest = cmax > kCmWide ? cmax - kCmWide : 0;
+  const int na = rest ? 1 : 2;
+  auto a_col = [&](int t) { return (uint32_t)((t & (na - 1)) * kCmWide); };
+  auto b_col = [&](int t) { return (uint32_t)(kCmWide + (t & 1) * rest); };
 
   if (warp == 0) {
-    // ------------------------------------------------------------ B producer
+    // ------------------------------------------------------------ table producer
     if (lane == 0) {
-      int st = 0;
+      int st = 0, prev = -1, nkb = 0, ncol = 0, col0 = 0;
       uint32_t ph = 0;
       int issued_phase[kCmMaxStages];
       for (int i = 0; i < kCmMaxStages; ++i) issued_phase[i] = -1;
       bool ok = true;
-      // resident table (one problem whose blocks all fit in the ring): each
-      // block is loaded once, into stage c nkb + q, and read by every tile
-      for (int i = blockIdx.x; ok && i < (resident ? min(ntiles, (int)blockIdx.x + 1) : ntiles); i += gridDim.x) {
-        const int4 tl = tiles[i];
-        const ProbDev& P = T.probs[tl.x];
-        const CUtensorMap* mt = T.tmaps + 2 * T.count + tl.x;
-        const int nkb = P.crt_kpad / 64, cw = P.crt_cw, nchunk = P.crt_nchunk, col0 = 32 * P.crt_gskip;
-        for (int c = 0; ok && c < nchunk; ++c) {
-          for (int q = 0; q < nkb; ++q) {
-            if (!mbar_wait(empty + st, ph ^ 1u, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
-            mbar_expect_tx(full + st, (uint32_t)cw * 128u);
-            tma_load_2d(sRing + st * stage_bytes, mt, smem_u32(full + st), q * 64, col0 + c * cw);
-            issued_phase[st] = (int)ph;
-            if (++st == stages) { st = 0; ph ^= 1u; }
-          }
+      CmWalk walk(segs);
+      for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
+        walk.seek(i);
+        if (walk.prob == prev && nkb <= stages) continue;     // this problem's table is in the ring
+        if (walk.prob != prev) {
+          const ProbDev& P = T.probs[walk.prob];
+          nkb = P.crt_kpad / 64;
+          col0 = 32 * P.crt_gskip;
+          ncol = P.crt_npad - col0;
+          prev = walk.prob;
+        }
+        const CUtensorMap* mt = T.tmaps + 2 * T.count + walk.prob;
+        for (int q = 0; q < nkb; ++q) {
+          if (!mbar_wait(empty + st, ph ^ 1u, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
+          mbar_expect_tx(full + st, (uint32_t)ncol * 128u);
+          for (int c = 0; c < ncol; c += 32)
+            tma_load_2d(sRing + st * stage_bytes + (uint32_t)c * 128u, mt, smem_u32(full + st), q * 64, col0 + c);
+          issued_phase[st] = (int)ph;
+          if (++st == stages) { st = 0; ph ^= 1u; }
         }
       }
       if (!ok) {
@@ -1389,231 +1432,223 @@ __global__ void __launch_bounds__(kCmThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int st = 0;
-      uint32_t ph = 0;
-      int next = 0, uses[2] = {0, 0}, vnext = 0, vuses[2] = {0, 0};
-      bool ok = true, any = false;
-      for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
-        const int4 tl = tiles[i];
-        const bool first = i == (int)blockIdx.x;
-        const ProbDev& P = T.probs[tl.x];
-        const int nkb = P.crt_kpad / 64, cw = P.crt_cw, nchunk = P.crt_nchunk, npad = P.crt_npad - 32 * P.crt_gskip;
-        const int nslot = P.crt_nslot, nvbuf = P.crt_nvbuf;
-        const uint32_t vcols = (uint32_t)P.crt_kpad / 2;
-        const int vb = nvbuf == 2 ? vnext : 0, vuse = vuses[vb]++;
-        vnext = nvbuf == 2 ? vnext ^ 1 : 0;
-        if (!mbar_wait(v_full + vb, (uint32_t)(vuse & 1), abort_flag, T.status, T.spin_limit)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t vbase = tmem + (uint32_t)vb * vcols;
-        for (int c = 0; ok && c < nchunk; ++c) {
-          const int s = nslot == 2 ? next : 0, use = uses[s]++;
-          next = nslot == 2 ? next ^ 1 : 0;
-          if (use > 0 && !mbar_wait(acc_free + s, (uint32_t)((use - 1) & 1), abort_flag, T.status, T.spin_limit)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const int ncol = min(cw, npad - c * cw);             // a multiple of 16
-          const uint32_t idesc = idesc_bf16(128, ncol);
-          const uint32_t d = tmem + (uint32_t)nvbuf * vcols + (uint32_t)(s * cw);
-          for (int q = 0; q < nkb; ++q) {
-            if (resident) st = c * nkb + q;
-            if ((!resident || first) && !mbar_wait(full + st, resident ? 0u : ph, abort_flag, T.status, T.spin_limit)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint64_t db = desc_sw128(sRing + st * stage_bytes);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_bf16_ta(d, vbase + (uint32_t)(32 * q + 8 * kk), db + 2 * kk, idesc, (q | kk) ? 1u : 0u);
-            any = true;
-            if (!resident) {
-              umma_commit(empty + st);
-              if (++st == stages) { st = 0; ph ^= 1u; }
-            }
-          }
-          if (ok) umma_commit(acc_full + s);
+    // the whole warp runs the loop, so that addresses and descriptors stay warp-uniform;
+    // one elected lane issues
+    {
+      const bool el = elect_one();
+      int st = 0, st0 = 0, prev = -1, nkb = 0, nks = 0, ca = 0, cb = 0;   // st0: first stage of a table that stays
+      uint32_t ph = 0, vph = 0;
+      int vs = 0, t = 0;
+      bool ok = true, any = false, stay = false;
+      auto wait = [&](uint64_t* bar, uint32_t parity) {
+        return ok = mbar_wait_warp(bar, parity, abort_flag, T.status, T.spin_limit);
+      };
+      CmWalk walk(segs);
+      for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x, ++t) {
+        walk.seek(i);
+        const bool fresh = !stay || walk.prob != prev;          // the table's stages are waited for
+        if (walk.prob != prev) {
+          const ProbDev& P = T.probs[walk.prob];
+          const int ncol = P.crt_npad - 32 * P.crt_gskip;
+          nkb = P.crt_kpad / 64;
+          nks = (2 * P.L + 15) / 16;                            // K steps of 16 that hold moduli
+          ca = min(ncol, kCmWide);
+          cb = ncol - ca;
+          stay = nkb <= stages;
+          prev = walk.prob;
         }
-        if (!ok) break;
-        umma_commit(v_free + vb);
+        if (fresh) st0 = st;
+        const bool last = !stay || i + (int)gridDim.x >= ntiles || i + (int)gridDim.x >= walk.end;
+        int sp = st0;
+        // the slots' previous tiles have been read
+        if (t >= na && !wait(a_free + ((t - na) & 1), (uint32_t)(((t - na) >> 1) & 1))) break;
+        if (t >= 2 && !wait(b_free + (t & 1), (uint32_t)(((t - 2) >> 1) & 1))) break;
+        tc_fence_after();
+        const uint32_t da = tmem + a_col(t), db = tmem + b_col(t);
+        const uint32_t ia = idesc_bf16(128, ca), ib = idesc_bf16(128, cb ? cb : 32);
+        for (int q = 0; q < nkb; ++q) {
+          if (fresh) {
+            if (!wait(full + st, ph)) break;
+            if (++st == stages) { st = 0; ph ^= 1u; }
+          }
+          if (!wait(v_full + vs, vph)) break;
+          tc_fence_after();
+          const uint64_t dv = desc_sw128(sV + (uint32_t)vs * kCmVBytes);
+          const uint64_t dt = desc_sw128(sRing + (uint32_t)sp * stage_bytes);
+          const uint64_t dr = desc_sw128(sRing + (uint32_t)sp * stage_bytes + kCmWide * 128u);
+          const int n = nks - 4 * q;
+          if (el) {
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+              if (kk < n) {
+                umma_bf16(da, dv + 2 * kk, dt + 2 * kk, ia, (q | kk) ? 1u : 0u);
+                if (cb) umma_bf16(db, dv + 2 * kk, dr + 2 * kk, ib, (q | kk) ? 1u : 0u);
+              }
+            }
+            umma_commit(v_free + vs);
+            if (last) umma_commit(empty + sp);
+          }
+          __syncwarp();
+          any = true;
+          if (++sp == stages) sp = 0;
+          if (++vs == kCmVSlots) { vs = 0; vph ^= 1u; }
+        }
+        if (ok && el) umma_commit(acc_full + (t & 1));
+        __syncwarp();
       }
       if (!ok && any) {
         // drain issued MMAs before TMEM is released
-        umma_commit(drain);
-        for (uint32_t t = 0; t < kSpinLimit && !mbar_try_wait(drain, 0u); ++t) {}
+        if (el) umma_commit(drain);
+        for (uint32_t s = 0; s < kSpinLimit && !mbar_try_wait(drain, 0u); ++s) {}
       }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------ v producer
     if (lane == 0) {
-      int uc = 0;
-      int issued_phase[kCmUSlots];
-      for (int i = 0; i < kCmUSlots; ++i) issued_phase[i] = -1;
+      int s = 0, L = 0, prev = -1;
+      uint32_t ph = 0;
+      int issued_phase[kCmMaxUSlots];
+      for (int i = 0; i < kCmMaxUSlots; ++i) issued_phase[i] = -1;
       bool ok = true;
+      CmWalk walk(segs);
       for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
-        const int4 tl = tiles[i];
-        const ProbDev& P = T.probs[tl.x];
-        const CUtensorMap* mu_ = T.tmaps + 3 * T.count + tl.x;
-        const int L = P.L;
-        for (int l0 = 0; l0 < L; l0 += kCmUMods, ++uc) {
-          const int s = uc % kCmUSlots, use = uc / kCmUSlots;
-          if (use > 0 && !mbar_wait(u_free + s, (uint32_t)((use - 1) & 1), abort_flag, T.status, T.spin_limit)) {
+        walk.seek(i);
+        if (walk.prob != prev) {
+          L = T.probs[walk.prob].L;
+          prev = walk.prob;
+        }
+        const CUtensorMap* mu_ = T.tmaps + 3 * T.count + walk.prob;
+        for (int l0 = 0; l0 < L; l0 += kCmUMods) {
+          if (!mbar_wait(u_free + s, ph ^ 1u, abort_flag, T.status, T.spin_limit)) {
             ok = false;
             break;
           }
           mbar_expect_tx(u_full + s, kCmUBytes);
-          tma_load_2d(sU + s * kCmUBytes, mu_, smem_u32(u_full + s), tl.y * 128, l0);
-          issued_phase[s] = use & 1;
+          tma_load_2d(sU + s * kCmUBytes, mu_, smem_u32(u_full + s), (i - walk.first) * 128, l0);
+          issued_phase[s] = (int)ph;
+          if (++s == uslots) { s = 0; ph ^= 1u; }
         }
       }
       if (!ok)
-        for (int s = 0; s < kCmUSlots; ++s)
-          if (issued_phase[s] >= 0)
-            for (uint32_t t = 0; t < kSpinLimit && !mbar_try_wait(u_full + s, (uint32_t)issued_phase[s]); ++t) {}
+        for (int q = 0; q < uslots; ++q)
+          if (issued_phase[q] >= 0)
+            for (uint32_t t = 0; t < kSpinLimit && !mbar_try_wait(u_full + q, (uint32_t)issued_phase[q]); ++t) {}
     }
+  } else if (warp < 3 + kCmBuildWarps) {
+    // ------------------------------------------------------------ V blocks
+    const int bt = threadIdx.x - 96;                  // 0 .. 255
+    const int row = bt & 127, half = bt >> 7;         // output row; moduli 16 half .. + 15 of the block
+    const uint16_t* s_u = reinterpret_cast<const uint16_t*>(sm + lay.u_off) + (16 * half) * 128 + row;
+    const uint32_t vrow = sV + (uint32_t)row * 128u;
+    int us = 0, vs = 0, L = 0, prev = -1;
+    uint32_t uph = 0, vph = 1;                        // vph: parity of the block's last release
+    bool ok = true, first_round = true;
+    CmWalk walk(segs);
+    for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
+      walk.seek(i);
+      if (walk.prob != prev) {
+        L = T.probs[walk.prob].L;
+        prev = walk.prob;
+      }
+      for (int l0 = 0; l0 < L; l0 += kCmUMods) {
+        ok = mbar_wait(u_full + us, uph, abort_flag, T.status, T.spin_limit);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const uint16_t* su = s_u + us * (kCmUMods * 128);
+        uint32_t pr[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pr[j] = su[j * 128];          // moduli past L arrive as zeros
+        __syncwarp();
+        if (lane == 0) mbar_arrive(u_free + us);
+        if (++us == uslots) { us = 0; uph ^= 1u; }
+        if (!first_round) ok = mbar_wait(v_free + vs, vph, abort_flag, T.status, T.spin_limit);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const uint32_t at = vrow + (uint32_t)vs * kCmVBytes;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)                                 // 16-byte chunk 4 half + c, 128-byte swizzle
+          st_shared_v4(at + (uint32_t)(((4 * half + c) ^ (row & 7)) << 4), bf16_halves7(pr[4 * c]),
+                       bf16_halves7(pr[4 * c + 1]), bf16_halves7(pr[4 * c + 2]), bf16_halves7(pr[4 * c + 3]));
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(v_full + vs);
+        if (++vs == kCmVSlots) { vs = 0; vph ^= 1u; first_round = false; }
+      }
+    }
+    if (!ok) *abort_flag = 1;
   } else {
-    // ------------------------------------------------------------ V columns + chunk epilogues
-    const int wk = warp - 3;
-    const int half = wk >> 2;                         // worker group 0..3
+    // ------------------------------------------------------------ group sums
+    const int sub = (warp - 3 - kCmBuildWarps) >> 2;  // groups sub, sub + 4, ...
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
     const uint32_t tlane = tmem + ((uint32_t)(quad * 32) << 16);
-    const uint16_t* s_u = reinterpret_cast<const uint16_t*>(sm + lay.u_off);
-    int next = 0, uses[2] = {0, 0}, uc = 0, vnext = 0, vuses[2] = {0, 0}, ecount = 0;
-    bool ok = true;
-    // V of tile i into its buffer: the group's v copies (c = h mod 4) as bf16
-    // 7-bit halves, and the group's part of the quotient sum
-    auto build = [&](int i) {
-      const int4 tl = tiles[i];
-      const ProbDev& P = T.probs[tl.x];
-      // the problem's fields in registers before the waits (their memory
-      // clobbers would reload them from global memory after every barrier)
-      const int L = P.L, nvbuf = P.crt_nvbuf;
-      const uint32_t vcols = (uint32_t)P.crt_kpad / 2;
-      const int vb = nvbuf == 2 ? vnext : 0, vuse = vuses[vb]++;
-      vnext = nvbuf == 2 ? vnext ^ 1 : 0;
-      // the buffer may be rewritten once every MMA of its previous tile is done
-      if (vuse > 0 && ok) ok = mbar_wait(v_free + vb, (uint32_t)((vuse - 1) & 1), abort_flag, T.status, T.spin_limit);
+    int t = 0, prev = -1, ngrp = 0;
+    bool ok = true, small = false;
+    int64_t up = 0, mn = 0;
+    uint32_t *qbase = nullptr, *abase = nullptr;
+    CmWalk walk(segs);
+    for (int i = blockIdx.x; i < ntiles; i += gridDim.x, ++t) {
+      walk.seek(i);
+      if (walk.prob != prev) {
+        const ProbDev& P = T.probs[walk.prob];
+        ngrp = (P.crt_npad - 32 * P.crt_gskip) >> 5;
+        small = 2 * P.L * 127 * 127 < (1 << 23);     // every column sum below 2^23
+        up = P.upitch;
+        mn = (int64_t)P.M * P.N;
+        qbase = P.crt_q;
+        abase = P.crt_alpha;
+        prev = walk.prob;
+      }
+      const int64_t idx = (int64_t)(i - walk.first) * 128 + row;
+      const bool valid = idx < mn;
+      ok = mbar_wait(acc_full + (t & 1), (uint32_t)((t >> 1) & 1), abort_flag, T.status, T.spin_limit);
       ok = __all_sync(0xffffffffu, ok);
-      if (!ok) return;
-      tc_fence_after();
-      const uint32_t vrow = tlane + (uint32_t)vb * vcols;
-      for (int l0 = 0; l0 < L; l0 += kCmUMods, ++uc) {
-        if ((uc & 3) != half) continue;             // another group's copy
-        const int s = uc % kCmUSlots, use = uc / kCmUSlots;
-        if (ok) ok = mbar_wait(u_full + s, (uint32_t)(use & 1), abort_flag, T.status, T.spin_limit);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) return;
-        const uint16_t* su = s_u + s * (kCmUMods * 128);
-        // pieces of 8 moduli in a rolled loop (small code), V columns
-        // l0 + 8 pc .. + 7 (zero beyond L)
-#pragma unroll 1
-        for (int pc = 0; pc < kCmUMods; pc += 8) {
-          const int lp = l0 + pc;
-          uint32_t pr[8];
-          if (lp + 8 <= L) {                          // a full piece: no bounds
-#pragma unroll
-            for (int j = 0; j < 8; ++j) pr[j] = bf16_halves7(su[(pc + j) * 128 + row]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int l = lp + j;
-              pr[j] = bf16_halves7(l < L ? (uint32_t)su[(pc + j) * 128 + row] : 0u);
-            }
-          }
-          tmem_st8(vrow + (uint32_t)lp, pr);
-        }
-        mbar_arrive(u_free + s);
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(v_full + vb);
-    };
-    // chunk epilogues of tile i: the tile's 32-column groups in turn over the
-    // four groups (rotated per tile)
-    auto epilogue = [&](int i) {
-      const int4 tl = tiles[i];
-      const ProbDev& P = T.probs[tl.x];
-      // columns from 32 crt_gskip on (the groups below are not formed); the
-      // group sums are stored from that group on
-      const int cw = P.crt_cw, nchunk = P.crt_nchunk, npad = P.crt_npad - 32 * P.crt_gskip, nslot = P.crt_nslot;
-      const uint32_t acc0 = (uint32_t)P.crt_nvbuf * ((uint32_t)P.crt_kpad / 2);
-      const bool small = 2 * P.L * 127 * 127 < (1 << 23);   // every column sum below 2^23
-      const int64_t idx = (int64_t)tl.y * 128 + row;
-      const bool valid = idx < (int64_t)P.M * P.N;
-      const int64_t up = P.upitch;
-      uint32_t* const qbase = P.crt_q;
-      for (int c = 0; c < nchunk; ++c) {
-        const int s = nslot == 2 ? next : 0, use = uses[s]++;
-        next = nslot == 2 ? next ^ 1 : 0;
-        if (ok) ok = mbar_wait(acc_full + s, (uint32_t)(use & 1), abort_flag, T.status, T.spin_limit);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) return;
-        tc_fence_after();
-        const uint32_t trow = tlane + acc0 + (uint32_t)(s * cw);
-        const int ncol = min(cw, npad - c * cw);             // columns written by the MMAs
-        const int gfirst = (half - c * (cw >> 5) - ecount) & 3;
-        for (int g = 32 * gfirst; g < cw; g += 128) {
-          uint64_t acc[7] = {0, 0, 0, 0, 0, 0, 0};
-          if (g < ncol) {
-            uint32_t y[32];
-            if (g + 32 <= ncol) {
-              tmem_ld32(trow + (uint32_t)g, y);
-            } else {                                  // 16 columns left: the rest are zero pieces
-              uint32_t y16[16];
-              tmem_ld16(trow + (uint32_t)g, y16);
-#pragma unroll
-              for (int q = 0; q < 16; ++q) y[q] = y16[q];
-#pragma unroll
-              for (int q = 16; q < 32; ++q) y[q] = 0u;
-            }
-            if (c * cw + g + 32 == npad) {
-              // the last group's columns 27..31 hold sum_k 128^k Y = sum_l v_l
-              // floor(2^28 / m_l): alpha~ = floor of it / 2^28, in {alpha - 1,
-              // alpha} (its error is below L 2^14 / 2^28); then they are cleared
-              uint64_t a = 0;
-#pragma unroll
-              for (int k = 4; k >= 0; --k) a = (a << 7) + f2u_exact24(y[27 + k]);
-              if (valid) P.crt_alpha[idx] = (uint32_t)(a >> 28);
-#pragma unroll
-              for (int k = 27; k < 32; ++k) y[k] = 0u;
-            }
-            if (small) crt_group_small<32>(y, acc);
-            else crt_group<32>(y, acc);
-          }
-          // group sum as 9 words: 7 word sums with carries, then the carry
-          uint32_t* qcol = qbase + (int64_t)((c * cw + g) >> 5) * 9 * up + (valid ? idx : 0);
-          uint64_t carry = 0;
-#pragma unroll
-          for (int k = 0; k < 7; ++k) {
-            const uint64_t x = acc[k] + carry;
-            if (valid) qcol[(int64_t)k * up] = (uint32_t)x;
-            carry = x >> 32;
-          }
-          if (valid) {
-            qcol[(int64_t)7 * up] = (uint32_t)carry;
-            qcol[(int64_t)8 * up] = (uint32_t)(carry >> 32);
-          }
-        }
-        tc_fence_before();
-        mbar_arrive(acc_free + s);
-      }
-      ++ecount;
-    };
-    // With two V buffers (uniform within a launch) the next tile's V is built
-    // before this tile's chunks are read, so its MMAs overlap the epilogue;
-    // that order waits for the MMAs of the tile before this one only.  With
-    // one buffer it would wait for this tile's MMAs, whose later chunks wait
-    // for this tile's epilogue: tiles then go strictly in turn.
-    const bool two = blockIdx.x < ntiles && T.probs[tiles[blockIdx.x].x].crt_nvbuf == 2;
-    if (two && blockIdx.x < ntiles) build(blockIdx.x);
-    for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
-      if (!two) build(i);
-      else if (i + (int)gridDim.x < ntiles) build(i + gridDim.x);
       if (!ok) break;
-      epilogue(i);
+      tc_fence_after();
+      bool gave_a = false;
+      for (int g = sub; g < ngrp; g += kCmEpiWarps / 4) {
+        if (!gave_a && g >= kCmWide / 32) {            // this warp's share of the first chunk is read
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(a_free + (t & 1));
+          gave_a = true;
+        }
+        uint32_t y[32];
+        tmem_ld32(tlane + (g < kCmWide / 32 ? a_col(t) + 32u * g : b_col(t) + 32u * g - kCmWide), y);
+        if (g == ngrp - 1) {
+          // columns 27..31 hold sum_k 128^k Y = sum_l v_l floor(2^28 / m_l):
+          // alpha~ = floor of it / 2^28, in {alpha - 1, alpha} (its error is
+          // below L 2^14 / 2^28); then they are cleared
+          uint64_t a = 0;
+#pragma unroll
+          for (int k = 4; k >= 0; --k) a = (a << 7) + f2u_exact24(y[27 + k]);
+          if (valid) abase[idx] = (uint32_t)(a >> 28);
+#pragma unroll
+          for (int k = 27; k < 32; ++k) y[k] = 0u;
+        }
+        uint64_t acc[7] = {0, 0, 0, 0, 0, 0, 0};
+        if (small) crt_group_small<32>(y, acc);
+        else crt_group<32>(y, acc);
+        // group sum as 9 words: 7 word sums with carries, then the carry
+        uint32_t* qcol = qbase + (int64_t)g * 9 * up + (valid ? idx : 0);
+        uint64_t carry = 0;
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+          const uint64_t x = acc[k] + carry;
+          if (valid) qcol[(int64_t)k * up] = (uint32_t)x;
+          carry = x >> 32;
+        }
+        if (valid) {
+          qcol[(int64_t)7 * up] = (uint32_t)carry;
+          qcol[(int64_t)8 * up] = (uint32_t)(carry >> 32);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (!gave_a) mbar_arrive(a_free + (t & 1));
+        mbar_arrive(b_free + (t & 1));
+      }
     }
     if (!ok) *abort_flag = 1;
   }
@@ -1693,55 +1728,32 @@ cudaError_t launch_crt_tc(const DevTables& t, int cls, const int32_t* tiles, int
   return cudaGetLastError();
 }
 
-// Chunk width of the tensor-core CRT sums: columns of Y per TMEM slot, a
-// multiple of 32, with V (kpad / 2 columns) and one or two slots within 512
-// columns.
-int crt_mm_chunk(int kpad, int npad, int* nslot) {
-  // two slots (the epilogue of one chunk overlaps the MMAs of the next)
-  // unless that leaves chunks narrower than 128 columns: one slot then, for
-  // MMAs of N >= 128 (narrow MMAs cost as much to issue as they compute)
-  const int need = (npad + 31) & ~31;
-  int cw2 = ((512 - kpad / 2) / 2) & ~31;
-  cw2 = cw2 > 256 ? 256 : cw2;
-  if (cw2 >= 128 || cw2 >= need) {
-    if (nslot) *nslot = 2;
-    return cw2 < need ? cw2 : need;
-  }
-  int cw1 = (512 - kpad / 2) & ~31;
-  cw1 = cw1 > 256 ? 256 : cw1;
-  if (nslot) *nslot = 1;
-  return cw1 < need ? cw1 : need;
+// Table stages of 64 k x cmax columns (at most kbmax, the K blocks of the longest
+// table) that fit beside the V ring and two v slots (0 if fewer than two do), and
+// the v slots that fit beside those: two 8 KB copies in flight per SM do not
+// cover the latency of the reads (1024^3 p = 256: 0.111 ms with two, 0.102 with
+// eight).
+static int crt_mm_stages(int cmax, int kbmax) {
+  int st = kbmax < 2 ? 2 : (kbmax < kCmMaxStages ? kbmax : kCmMaxStages);
+  while (st >= 2 && CmLayout((uint32_t)cmax * 128u, st, kCmMinUSlots).total > 227u * 1024u) --st;
+  return st < 2 ? 0 : st;
 }
-
-int crt_mm_smem_bytes(int cw_max, int lmax, int* stages) {
-  // the deepest B ring (2 to kCmMaxStages stages of cw_max columns) that fits
-  const uint32_t sb = (uint32_t)cw_max * 128u;
-  for (int st = kCmMaxStages; st >= 2; --st) {
-    const int bytes = (int)CmLayout(sb, st, lmax).total;
-    if (bytes <= 227 * 1024) {
-      if (stages) *stages = st;
-      return bytes;
-    }
-  }
-  if (stages) *stages = 0;
-  return -1;
+static int crt_mm_uslots(int cmax, int stages) {
+  int us = kCmMaxUSlots;
+  while (us > kCmMinUSlots && CmLayout((uint32_t)cmax * 128u, stages, us).total > 227u * 1024u) --us;
+  return us;
 }
+bool crt_mm_fits(int cols) { return cols <= kCmCols && crt_mm_stages(cols, kCmMaxStages) >= 2; }
 
-// blocks_one: the table blocks of a tile (K blocks x chunks) when every tile
-// of the launch belongs to one problem, else 0; where they fit in the ring
-// the table stays resident (loaded once per CTA).
-cudaError_t launch_crt_mm(const DevTables& t, const int32_t* tiles, int ntiles, int cw_max, int grid,
-                          int blocks_one, cudaStream_t s) {
+cudaError_t launch_crt_mm(const DevTables& t, const int32_t* segs, int ntiles, int cmax, int kbmax, int sms,
+                          cudaStream_t s) {
   if (ntiles == 0) return cudaSuccess;
-  int stages = 0;
-  const int smem = crt_mm_smem_bytes(cw_max, t.lmax, &stages);
-  if (smem < 0) return cudaErrorInvalidValue;
-  const int g = ntiles < grid ? ntiles : grid;
-  const int4* tl = reinterpret_cast<const int4*>(tiles);
-  if (blocks_one > 0 && blocks_one <= stages)
-    k_crt_mm<true><<<g, kCmThreads, smem, s>>>(t, tl, ntiles, (uint32_t)cw_max * 128u, stages);
-  else
-    k_crt_mm<false><<<g, kCmThreads, smem, s>>>(t, tl, ntiles, (uint32_t)cw_max * 128u, stages);
+  const int stages = crt_mm_stages(cmax, kbmax);
+  if (stages == 0) return cudaErrorInvalidValue;
+  const int us = crt_mm_uslots(cmax, stages);
+  const uint32_t stage_bytes = (uint32_t)cmax * 128u;
+  k_crt_mm<<<ntiles < sms ? ntiles : sms, kCmThreads, CmLayout(stage_bytes, stages, us).total, s>>>(
+      t, reinterpret_cast<const int4*>(segs), ntiles, stage_bytes, stages, us, cmax);
   return cudaGetLastError();
 }
 
@@ -1776,9 +1788,7 @@ cudaError_t launch_crt_fin_short(const DevTables& t, int cls, const int32_t* blk
 }
 
 cudaError_t init_crt_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_crt_mm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_crt_mm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  cudaError_t e = cudaFuncSetAttribute(k_crt_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_crt_fin_long, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   if (e == cudaSuccess) e = crt1_attr<8>();

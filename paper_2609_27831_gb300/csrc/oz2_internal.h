@@ -85,20 +85,18 @@ struct ProbDev {
   int32_t crt_kpad;      // tensor-core CRT: K = 2L padded to a multiple of 64
   int32_t crt_npad;      // tensor-core CRT: 7-bit pieces of S padded to a multiple of 16
   int32_t crt_np;        // tensor-core CRT: 7-bit pieces of S (columns of Y)
-  int32_t crt_nvbuf;     // crt_mode 2: V buffers in TMEM (2 where kpad + nslot cw <= 512)
+  int32_t pad2;
   int64_t upitch;        // row pitch of u [L][upitch]: M*N rounded up to a multiple of 8
   int32_t res_mode;      // 0: residues on the CUDA cores; 1: byte GEMM on the tensor cores;
                          // 2: the byte GEMM, warp-specialised (bytes in TMEM, table streamed)
   int32_t res_kpad;      // tensor-core residues: bytes of a (t+1)-bit integer, padded to 64
   int32_t res_npad;      // tensor-core residues: table rows L1 + 2 (L - L1), padded to 16
-  int32_t crt_nchunk;    // crt_mode 2: chunks of crt_cw columns of Y
-  int32_t crt_cw;        // crt_mode 2: columns of Y per chunk (a multiple of 32)
   uint32_t* crt_q;       // crt_mode 2: group sums Q_g as [ngrp][9][upitch] words
   uint32_t* crt_alpha;   // crt_mode 2: quotient estimates alpha~ [upitch]
-  int32_t crt_ngrp;      // crt_mode 2: groups of 32 columns, nchunk cw / 32
+  int32_t crt_ngrp;      // crt_mode 2: groups of 32 columns formed
   int32_t res_cw;        // res_mode 2: columns of Y per chunk (a multiple of 32)
   int32_t res_nchunk;    // res_mode 2: chunks
-  int32_t crt_nslot;     // crt_mode 2: TMEM accumulator slots (1 or 2)
+  int32_t pad3;
   int32_t res_nabuf;     // res_mode 2: byte buffers (A) in TMEM (2 or 4)
   int32_t u_map;         // 1: tensor map 5 * count + i stores v_l tiles (N a multiple of 8)
   int32_t* dbg_prods;    // optional (K within one chunk): [G][M][N] exact plane sums before reduction
@@ -181,13 +179,13 @@ cudaError_t launch_crt(const DevTables& t, int cls, const int32_t* blk_list, int
 cudaError_t launch_crt_tc(const DevTables& t, int cls, const int32_t* tiles, int ntiles, int kpad_max,
                           int npad_max, int lmax, int sms, cudaStream_t s);
 int crt_tc_smem_bytes(int cls, int kpad_max, int npad_max, int lmax, int nbuf);
-// Tensor-core CRT sums of any length (crt_mode 2): tiles of 128 outputs
-// {problem, tile}; R digits to the workspace.  Then the finish of long
-// accumulators (> 40 digits), blocks of 128 outputs {problem, block}.
-cudaError_t launch_crt_mm(const DevTables& t, const int32_t* tiles, int ntiles, int cw_max, int grid,
-                          int blocks_one, cudaStream_t s);
-int crt_mm_chunk(int kpad, int npad, int* nslot);
-int crt_mm_smem_bytes(int cw_max, int lmax, int* stages);
+// Tensor-core CRT sums of any length (crt_mode 2): runs of tiles of 128 outputs
+// {problem, first tile, end, 0}, cmax and kbmax the most formed columns and K
+// blocks of 64; group sums to the workspace.  Then the finish of long accumulators, blocks of 128
+// outputs {problem, block}.
+cudaError_t launch_crt_mm(const DevTables& t, const int32_t* segs, int ntiles, int cmax, int kbmax, int sms,
+                          cudaStream_t s);
+bool crt_mm_fits(int cols);
 // the finish of one-lane classes after the tensor-core sums (the host uses it up to 24 digits)
 cudaError_t launch_crt_fin_short(const DevTables& t, int cls, const int32_t* blk, int nblk, cudaStream_t s);
 int crt_finish_long_smem(int dmax, int nlmax);
