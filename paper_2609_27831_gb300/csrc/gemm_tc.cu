@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kStages + 5);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 6);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int cta = blockIdx.x;
   const int ubeg = T.cta_begin[cta], uend = T.cta_begin[cta + 1];
 
@@ -90,8 +90,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------------------------------------------ producer
+    const bool el = elect_one();
     JobIter it;
     it.init(&T, ubeg, uend);
     Job j;
@@ -107,11 +108,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
       const int k0 = j.chunk * P.kchunk;
       const int k1 = min(P.K, k0 + P.kchunk);
       for (int k = k0; k < k1; k += kBK) {
-        if (!mbar_wait(empty + st, ph ^ 1u, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
-        mbar_expect_tx(full + st, kStageBytes);
+        ok = mbar_wait_warp(empty + st, ph ^ 1u, abort_flag, T.status, T.spin_limit);
+        if (!ok) break;
         const uint32_t sa = base + st * kStageBytes;
-        tma_load_3d(sa, ma, smem_u32(full + st), k, j.u.tm * kBM, j.plane);
-        tma_load_3d(sa + kTileABytes, mb, smem_u32(full + st), k, j.u.tn * kBN, j.plane);
+        if (el) {
+          mbar_expect_tx(full + st, kStageBytes);
+          tma_load_3d(sa, ma, smem_u32(full + st), k, j.u.tm * kBM, j.plane);
+          tma_load_3d(sa + kTileABytes, mb, smem_u32(full + st), k, j.u.tn * kBN, j.plane);
+        }
+        __syncwarp();
         issued_phase[st] = (int)ph;
         if (++st == kStages) { st = 0; ph ^= 1u; }
       }
@@ -124,8 +129,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
+    // The whole warp runs the loop, so that addresses and descriptors stay
+    // warp-uniform; one elected lane issues; the producer likewise.
+    // (In a single-lane branch and now, plane GEMMs: 8192^3 p = 53 16.3 and
+    // 15.6 ms, 4096^3 p = 2048 73.5 and 70.)
+    const bool el = elect_one();
     JobIter it;
     it.init(&T, ubeg, uend);
     Job j;
@@ -140,33 +150,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
       const int k0 = j.chunk * P.kchunk;
       const int k1 = min(P.K, k0 + P.kchunk);
       if (uses[s] > 0) {
-        if (!mbar_wait(slot_free + s, (uint32_t)((uses[s] - 1) & 1), abort_flag, T.status, T.spin_limit)) { ok = false; break; }
+        ok = mbar_wait_warp(slot_free + s, (uint32_t)((uses[s] - 1) & 1), abort_flag, T.status, T.spin_limit);
+        if (!ok) break;
       }
       ++uses[s];
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(s * kBN);
       bool acc = !j.first;
       for (int k = k0; k < k1; k += kBK) {
-        if (!mbar_wait(full + st, ph, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
+        ok = mbar_wait_warp(full + st, ph, abort_flag, T.status, T.spin_limit);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t sa = base + st * kStageBytes;
         const uint64_t da = desc_sw128(sa);
         const uint64_t db = desc_sw128(sa + kTileABytes);
+        if (el) {
 #pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk) {
-          umma(d, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), acc ? 1u : 0u);
-          acc = true;
+          for (int kk = 0; kk < kBK / 16; ++kk)
+            umma(d, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), (acc || kk) ? 1u : 0u);
+          umma_commit(empty + st);
         }
-        umma_commit(empty + st);
-        any = true;
+        __syncwarp();
+        acc = any = true;
         if (++st == kStages) { st = 0; ph ^= 1u; }
       }
       if (!ok) break;
-      umma_commit(slot_full + s);
+      if (el) umma_commit(slot_full + s);
+      __syncwarp();
     }
     if (!ok && any) {
       // drain issued MMAs before TMEM is released
-      umma_commit(drain);
+      if (el) umma_commit(drain);
       for (uint32_t t = 0; t < kSpinLimit && !mbar_try_wait(drain, 0); ++t) {}
     }
   } else if (warp >= 2) {

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThreads2, 1) k_gemm_tc2(const __grid_constant
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kStages2 + 5);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages2 + 6);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int pair = blockIdx.x >> 1;
@@ -140,8 +140,9 @@ __global__ void __launch_bounds__(kThreads2, 1) k_gemm_tc2(const __grid_constant
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------------------------------------------ producer (both CTAs)
+    const bool el = elect_one();
     JobIter it;
     it.init(&T, ubeg, uend);
     Job j;
@@ -160,12 +161,16 @@ __global__ void __launch_bounds__(kThreads2, 1) k_gemm_tc2(const __grid_constant
       const int arow = j.u.tm * 256 + (int)rank * kRows;
       const int brow = j.u.tn * 256 + (int)rank * kRows;
       for (int k = k0; k < k1; k += kBK) {
-        if (!mbar_wait(empty + st, ph ^ 1u, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
-        if (leader) mbar_expect_tx(full + st, 2u * kStageBytes2);
+        ok = mbar_wait_warp(empty + st, ph ^ 1u, abort_flag, T.status, T.spin_limit);
+        if (!ok) break;
         const uint32_t sa = base + st * kStageBytes2;
         const uint32_t fb = full_leader0 + (uint32_t)(st * 8);
-        tma_load_3d_pair(sa, ma, fb, k, arow, j.plane);
-        tma_load_3d_pair(sa + kTileBytes, mb, fb, k, brow, j.plane);
+        if (el) {
+          if (leader) mbar_expect_tx(full + st, 2u * kStageBytes2);
+          tma_load_3d_pair(sa, ma, fb, k, arow, j.plane);
+          tma_load_3d_pair(sa + kTileBytes, mb, fb, k, brow, j.plane);
+        }
+        __syncwarp();
         issued_phase[st] = (int)ph;
         if (++st == kStages2) { st = 0; ph ^= 1u; }
       }
@@ -184,8 +189,13 @@ __global__ void __launch_bounds__(kThreads2, 1) k_gemm_tc2(const __grid_constant
         for (int t = 0; t < 100; ++t) __nanosleep(1000);
       }
     }
-  } else if (warp == 1 && lane == 0 && leader) {
+  } else if (warp == 1 && leader) {
     // ------------------------------------------------------------ MMA issuer (leader)
+    // The whole warp runs the loop, so that addresses and descriptors stay
+    // warp-uniform; one elected lane issues; the producer likewise.
+    // (In a single-lane branch and now, plane GEMMs: 1024^3 p = 256 0.160
+    // and 0.146 ms, p = 2048 1.22 and 1.12.)
+    const bool el = elect_one();
     JobIter it;
     it.init(&T, ubeg, uend);
     Job j;
@@ -200,38 +210,40 @@ __global__ void __launch_bounds__(kThreads2, 1) k_gemm_tc2(const __grid_constant
       const int k0 = j.chunk * P.kchunk;
       const int k1 = min(P.K, k0 + P.kchunk);
       if (uses[s] > 0) {
-        if (!mbar_wait(slot_free + s, (uint32_t)((uses[s] - 1) & 1), abort_flag, T.status, T.spin_limit)) {
-          ok = false;
-          break;
-        }
+        ok = mbar_wait_warp(slot_free + s, (uint32_t)((uses[s] - 1) & 1), abort_flag, T.status, T.spin_limit);
+        if (!ok) break;
       }
       ++uses[s];
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(s * kBN);
       bool acc = !j.first;
       for (int k = k0; k < k1; k += kBK) {
-        if (!mbar_wait(full + st, ph, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
+        ok = mbar_wait_warp(full + st, ph, abort_flag, T.status, T.spin_limit);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t sa = base + st * kStageBytes2;
         const uint64_t da = desc_sw128(sa);
         const uint64_t db = desc_sw128(sa + kTileBytes);
+        if (el) {
 #pragma unroll
-        for (int kk = 0; kk < kBK / 16; ++kk) {
-          umma_pair(d, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), acc ? 1u : 0u);
-          acc = true;
+          for (int kk = 0; kk < kBK / 16; ++kk)
+            umma_pair(d, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), (acc || kk) ? 1u : 0u);
+          commit_pair(empty + st);
         }
-        commit_pair(empty + st);
-        any = true;
+        __syncwarp();
+        acc = any = true;
         if (++st == kStages2) { st = 0; ph ^= 1u; }
       }
       if (!ok) break;
-      commit_pair(slot_full + s);
+      if (el) commit_pair(slot_full + s);
+      __syncwarp();
     }
     if (!ok && any) {
       // drain issued MMAs before TMEM is released
-      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_u32(drain))
-                   : "memory");
+      if (el)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                         smem_u32(drain))
+                     : "memory");
       for (uint32_t t = 0; t < kSpinLimit && !mbar_try_wait(drain, 0); ++t) {}
     }
   } else if (warp >= 2) {
