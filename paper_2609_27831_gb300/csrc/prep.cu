@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kRmThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(acc_full + 13);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 13) + 1;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   {
     float4* w_mc = reinterpret_cast<float4*>(sm + lay.mc_off);
     for (int l = threadIdx.x; l < T.lmax; l += kRmThreads) {
@@ -865,11 +865,17 @@ __global__ void __launch_bounds__(kRmThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // the whole warp runs the loop, so that addresses and descriptors stay warp-uniform;
+    // one elected lane issues (1024^3 p = 2048: 1.80 ms from a single-lane branch, 1.65 so)
+    {
+      const bool el = elect_one();
       int st = 0;
       uint32_t ph = 0;
       int ck = 0, tcount = 0;
       bool ok = true, any = false;
+      auto wait = [&](uint64_t* bar, uint32_t parity) {
+        return ok = mbar_wait_warp(bar, parity, abort_flag, T.status, T.spin_limit);
+      };
       for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x, ++tcount) {
         const int4 tl = tiles[i];
         const ProbDev& P = T.probs[tl.x];
@@ -877,37 +883,39 @@ __global__ void __launch_bounds__(kRmThreads, 1)
         const uint32_t acols = (uint32_t)P.res_kpad / 2;
         const int nabuf = P.res_nabuf;
         const int ab = tcount % nabuf, ause = tcount / nabuf;
-        if (!mbar_wait(a_full + ab, (uint32_t)(ause & 1), abort_flag, T.status, T.spin_limit)) { ok = false; break; }
+        if (!wait(a_full + ab, (uint32_t)(ause & 1))) break;
         tc_fence_after();
         const uint32_t abase = tmem + (uint32_t)ab * acols;
         for (int c = 0; ok && c < nchunk; ++c, ++ck) {
           const int s = ck & 1, use = ck >> 1;
-          if (use > 0 && !mbar_wait(acc_free + s, (uint32_t)((use - 1) & 1), abort_flag, T.status, T.spin_limit)) {
-            ok = false;
-            break;
-          }
+          if (use > 0 && !wait(acc_free + s, (uint32_t)((use - 1) & 1))) break;
           tc_fence_after();
           const int ncol = min(cw, npad - c * cw);             // a multiple of 16
           const uint32_t idesc = idesc_f16(128, ncol);             // f16 bytes and f16 table
           const uint32_t d = tmem + (uint32_t)nabuf * acols + (uint32_t)(s * cw);
           for (int q = 0; q < nkb; ++q) {
-            if (!mbar_wait(full + st, ph, abort_flag, T.status, T.spin_limit)) { ok = false; break; }
+            if (!wait(full + st, ph)) break;
             tc_fence_after();
             const uint64_t db = desc_sw128(sRing + st * stage_bytes);
+            if (el) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_bf16_ta(d, abase + (uint32_t)(32 * q + 8 * kk), db + 2 * kk, idesc, (q | kk) ? 1u : 0u);
-            umma_commit(empty + st);
+              for (int kk = 0; kk < 4; ++kk)
+                umma_bf16_ta(d, abase + (uint32_t)(32 * q + 8 * kk), db + 2 * kk, idesc, (q | kk) ? 1u : 0u);
+              umma_commit(empty + st);
+            }
+            __syncwarp();
             any = true;
             if (++st == stages) { st = 0; ph ^= 1u; }
           }
-          if (ok) umma_commit(acc_full + s);
+          if (ok && el) umma_commit(acc_full + s);
+          __syncwarp();
         }
         if (!ok) break;
-        umma_commit(a_free + ab);
+        if (el) umma_commit(a_free + ab);
+        __syncwarp();
       }
       if (!ok && any) {
-        umma_commit(drain);
+        if (el) umma_commit(drain);
         for (uint32_t t = 0; t < kSpinLimit && !mbar_try_wait(drain, 0u); ++t) {}
       }
     }
