@@ -894,6 +894,48 @@ __device__ __forceinline__ uint32_t sub_chain(const uint32_t (&a)[N], const uint
   return t & 1u;
 }
 
+// Digits of R = sum_l v_l M_l + alpha~ (2^(32 D) - P) of output sidx, by a
+// converged warp, into lane src's Rv, 64 digits at a time: lane j sums the digits
+// d = j mod 32 over every modulus (the v_l of 32 moduli read at once, one per
+// lane; the digits of M_l coalesced across the lanes, eight moduli in flight; each
+// sum is below L 2^46 + alpha~ 2^32 < 2^56), then every lane runs the same carry
+// chain over the digits, each fetched from its lane.  Few outputs need it, but
+// each is one warp's serial work in the launch's tail: with one v_l and one row of
+// M_l in flight it stretched the finish of 1024^3 p = 2048 to 0.65 ms (0.32 so).
+// A function of its own and 64 digits at a time (all at once: 96 registers) keep
+// the common path at 72 registers, which p = 512 and 1024 need (0.182 and 0.205 ms
+// at 72 and 96, 1536 x 1093 outputs of p = 512).
+__device__ __noinline__ void rebuild_digits(const ProbDev& P, const uint32_t* Mdig, const uint32_t* s_negP,
+                                            int64_t sidx, uint32_t alpha, int src, uint32_t* Rv) {
+  const int lane = threadIdx.x & 31, D = P.D32, L = P.L, DS = P.DS;
+  const uint16_t* u = P.u + sidx;
+  uint64_t c = 0;
+#pragma unroll 1
+  for (int d0 = 0; d0 < D; d0 += 64) {
+    const bool in0 = d0 + lane < D, in1 = d0 + 32 + lane < D;
+    uint64_t a0 = in0 ? (uint64_t)alpha * s_negP[d0 + lane] : 0ull;
+    uint64_t a1 = in1 ? (uint64_t)alpha * s_negP[d0 + 32 + lane] : 0ull;
+    const uint32_t* ml = Mdig + d0 + lane;
+#pragma unroll 1
+    for (int l0 = 0; l0 < L; l0 += 32) {
+      const uint32_t vl = l0 + lane < L ? __ldg(u + (int64_t)(l0 + lane) * P.upitch) : 0u;
+      const int n = min(32, L - l0);
+#pragma unroll 8
+      for (int i = 0; i < n; ++i, ml += DS) {
+        const uint64_t v = __shfl_sync(kFull, vl, i);
+        if (in0) a0 += v * __ldg(ml);
+        if (in1) a1 += v * __ldg(ml + 32);
+      }
+    }
+#pragma unroll 1
+    for (int i = 0; i < 64 && d0 + i < D; ++i) {
+      const uint64_t x = __shfl_sync(kFull, i < 32 ? a0 : a1, i & 31) + c;
+      c = x >> 32;
+      if (lane == src) Rv[d0 + i] = (uint32_t)x;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kFinThreads) k_crt_fin_long(DevTables T, const int4* __restrict__ blk) {
   extern __shared__ __align__(16) uint32_t sf[];
   const int4 b = blk[blockIdx.x];
@@ -1081,45 +1123,14 @@ __global__ void __launch_bounds__(kFinThreads) k_crt_fin_long(DevTables T, const
     }
   }
   // R from v_l for each lane whose fast form did not stand while the lower
-  // group sums were not formed, one such lane at a time by the whole warp:
-  // lane j sums the digits d = j mod 32 over every modulus (the digits of
-  // M_l read coalesced across the lanes, v_l one broadcast word; each sum is
-  // below L 2^46 + alpha~ 2^32 < 2^56), then every lane runs the same carry
-  // chain over the digits (each fetched from its lane) and the owner keeps
-  // them.
+  // group sums were not formed, one such lane at a time by the whole warp
   {
     const unsigned need = __ballot_sync(0xffffffffu, valid && !fast && gsk > 0);
-    const int L = P.L, DS = P.DS;
     for (unsigned m = need; m; m &= m - 1) {
       const int src = __ffs(m) - 1;
       const int64_t sidx = __shfl_sync(0xffffffffu, idx, src);
       const uint32_t salpha = __shfl_sync(0xffffffffu, alpha, src);
-      constexpr int kJ = kCrtSkipMaxDigits / 32;
-      uint64_t acc[kJ];
-#pragma unroll
-      for (int j = 0; j < kJ; ++j) {
-        const int d = 32 * j + lane;
-        acc[j] = d < D ? (uint64_t)salpha * s_negP[d] : 0ull;
-      }
-      for (int l = 0; l < L; ++l) {
-        const uint64_t v = __ldg(P.u + (int64_t)l * up + sidx);
-        const uint32_t* ml = cv.Mdig + (int64_t)l * DS;
-#pragma unroll
-        for (int j = 0; j < kJ; ++j) {
-          const int d = 32 * j + lane;
-          if (32 * j < D && d < D) acc[j] += v * __ldg(ml + d);
-        }
-      }
-      uint64_t c = 0;
-#pragma unroll
-      for (int j = 0; j < kJ; ++j) {
-        if (32 * j >= D) break;
-        for (int ln = 0; ln < 32 && 32 * j + ln < D; ++ln) {
-          const uint64_t x = __shfl_sync(0xffffffffu, acc[j], ln) + c;
-          c = x >> 32;
-          if (lane == src) Rv[32 * j + ln] = (uint32_t)x;
-        }
-      }
+      rebuild_digits(P, cv.Mdig, s_negP, sidx, salpha, src, Rv);
       if (lane == src) from_v = true;
     }
   }
