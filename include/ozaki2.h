@@ -108,11 +108,12 @@ typedef struct {
                      32 <= L <= 448 and M N >= 128 (CUDA cores otherwise);
                      3: the CRT on the CUDA cores only */
   int res_engine; /* 0: automatic (default): engine 2 for integers of more than 72 bytes
-                     (p above about 550), CUDA cores otherwise; 1: residues as an exact bf16
+                     (p above about 550), engine 3 otherwise; 1: residues as an exact bf16
                      GEMM of the bytes of a_hat with a table of centered 2^(8b) mod m on the
-                     tensor cores where the table has <= 256 rows and <= 256 bytes (CUDA cores
+                     tensor cores where the table has <= 256 rows and <= 256 bytes (engine 3
                      otherwise); 2: the same GEMM, warp-specialised (bytes in tensor memory, table
-                     streamed), for integers of up to 448 bytes; 3: CUDA cores only */
+                     streamed), for integers of up to 448 bytes; 3: in registers, warp-level products of
+                     the bytes up to 72 of them, dp4a on the CUDA cores beyond */
   int plane_group; /* residue planes streamed through the workspace in groups of consecutive
                      moduli (single-product plans with the tensor-core engine and the grouped
                      schedule; batched plans ignore it): 0 automatic (default): one group while
@@ -139,7 +140,7 @@ typedef struct {
   size_t workspace_bytes;
   int crt_mode;     /* CRT path of problem 0: 0 CUDA cores, 1 tensor-core column sums in one
                        kernel, 2 tensor-core sums of any length plus the finish (see crt_engine) */
-  int res_mode;     /* residue path of problem 0: 0 CUDA cores, 1 or 2 tensor cores (res_engine) */
+  int res_mode;     /* residue path of problem 0: 0 in registers, 1 or 2 byte GEMM (res_engine) */
   int plane_groups; /* modulus groups the planes of problem 0 are streamed in (1: not streamed) */
   int group_planes; /* planes of the largest group (= G when not streamed) */
   int gemm_tile;    /* plane GEMM tile in use: 1 (128 x 256, one SM) or 2 (256 x 256, CTA pairs) */

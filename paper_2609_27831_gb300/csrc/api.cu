@@ -827,7 +827,7 @@ struct TableImage {
          o_srows = 0, o_scols = 0, o_simt = 0, o_s8 = 0, o_status = 0;
   size_t o_res[6] = {0}, o_crt[kCrtClassCount] = {0};
   int n_srows = 0, n_scols = 0, n_simt = 0, n_s8 = 0, n_res[6] = {0}, n_crt[kCrtClassCount] = {0};
-  int res_l[6] = {0}, crt_l[kCrtClassCount] = {0};
+  int res_l[6] = {0}, res_tiles[6] = {0}, crt_l[kCrtClassCount] = {0};
   int grid = 0;
   // tensor-core CRT: tile lists per one-lane class, table offsets per CRT key
   size_t o_tct[9] = {0};
@@ -1063,7 +1063,10 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
         for (int64_t k = 0; k < h.K; k += 32 * residue_class_ept(h.res_cls))
           res[h.res_cls].push_back(make_int4(pi, side, (int)r, (int)k));
     }
-    if (h.res_mode == 0 && own_planes) ti.res_l[h.res_cls] = std::max(ti.res_l[h.res_cls], h.L);
+    if (h.res_mode == 0 && own_planes) {
+      ti.res_l[h.res_cls] = std::max(ti.res_l[h.res_cls], h.L);
+      ti.res_tiles[h.res_cls] = std::max(ti.res_tiles[h.res_cls], residue_tiles(h.L, h.L1));
+    }
     if (h.no_crt) {
       // no CRT for this problem
     } else if (h.crt_mode == 1) {
@@ -1218,7 +1221,7 @@ static void install_table_image(ozaki2_plan_s* pl, const TableImage& ti, uint8_t
   d.s8 = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_s8), ti.n_s8, 0, 0};
   for (int i = 0; i < 6; ++i)
     d.res[i] = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_res[i]), ti.n_res[i],
-                       ti.res_l[i] * (residue_class_w16(i) + 4) * 4, ti.res_l[i], ti.na_res[i]};
+                       residue_class_smem(i, ti.res_l[i], ti.res_tiles[i]), ti.res_l[i], ti.na_res[i]};
   for (int i = 0; i < 9; ++i) {
     d.tct[i] = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_tct[i]), ti.n_tct[i], ti.tct_kpad[i], ti.tct_l[i]};
     d.tct_npad[i] = ti.tct_npad[i];

@@ -87,7 +87,7 @@ struct ProbDev {
   int32_t crt_np;        // tensor-core CRT: 7-bit pieces of S (columns of Y)
   int32_t pad2;
   int64_t upitch;        // row pitch of u [L][upitch]: M*N rounded up to a multiple of 8
-  int32_t res_mode;      // 0: residues on the CUDA cores; 1: byte GEMM on the tensor cores;
+  int32_t res_mode;      // 0: residues in registers (warp-level products, dp4a beyond 72 bytes); 1: byte GEMM;
                          // 2: the byte GEMM, warp-specialised (bytes in TMEM, table streamed)
   int32_t res_kpad;      // tensor-core residues: bytes of a (t+1)-bit integer, padded to 64
   int32_t res_npad;      // tensor-core residues: table rows L1 + 2 (L - L1), padded to 16
@@ -227,7 +227,9 @@ int plan_run(ozaki2_plan pl, const ozaki2_problem* q, void* ws, size_t ws_bytes,
 // Residue kernel W16 classes and CRT lane-group classes (host picks per problem).
 int residue_class_for(int w16);        // -> class index, or -1
 int residue_class_w16(int cls);
-int residue_class_ept(int cls);       // elements per thread of that class (block: 32 EPT k x 8 lines)
+int residue_class_ept(int cls);       // k of a block of that class / 32 (8 lines)
+int residue_tiles(int L, int L1);     // 16-row tiles of the moduli (classes up to 72 bytes)
+int residue_class_smem(int cls, int lmax, int tiles);   // dynamic shared memory
 constexpr int kCrtClassCount = 12;
 int crt_class_for(int d32);            // -> class index, or -1
 int crt_class_elems_per_block(int cls);

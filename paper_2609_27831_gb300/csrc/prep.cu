@@ -89,7 +89,6 @@ __device__ __forceinline__ uint32_t sig_word(const uint32_t* __restrict__ limbs3
 // modulus's table row ahead of them (about 1 % at 1024^3, p = 256).
 __device__ __forceinline__ void st_plane(uint16_t* p, uint32_t bits) { __stcg(reinterpret_cast<unsigned short*>(p), (unsigned short)bits); }
 __device__ __forceinline__ void st_plane2(uint16_t* p, uint32_t v) { __stcg(reinterpret_cast<unsigned int*>(p), v); }
-__device__ __forceinline__ void st_plane4(uint16_t* p, uint2 v) { __stcg(reinterpret_cast<uint2*>(p), v); }
 
 // Bytes b0, b1 (sel 0x5140) or b2, b3 (sel 0x7362) of x as an f16 pair (low
 // half first): the byte permute puts each byte under the f16 exponent bits of
@@ -118,22 +117,19 @@ __device__ __forceinline__ int centered(uint32_t r, uint32_t m, bool neg) {
 
 // Words of |a_hat| = floor(sig 2^sh) + rnd for one element (32 bits each,
 // the round-half-even increment carried through the words).  A zero element
-// gives zero words.
-template <int W32>
-__device__ __forceinline__ void element_words(const uint64_t* __restrict__ limbs, int64_t ps, int64_t off,
-                                              int nl, int exp_el, int e_line, int t, uint32_t (&wd)[W32]) {
+// gives zero words.  limb(j) is limb j of the significand, 0 outside [0, nl).
+template <int W32, class Limb>
+__device__ __forceinline__ void element_words(Limb limb, int nl, int exp_el, int e_line, int t,
+                                              uint32_t (&wd)[W32]) {
 #pragma unroll
   for (int w = 0; w < W32; ++w) wd[w] = 0u;
   const int sh = exp_el - e_line + t - 64 * nl;   // <= t - 64 nl
   const int B = 64 - sh;                          // bit of S = sig 2^64 that is bit 0 of the magnitude
   if (B - 1 >= 64 * nl + 64) return;              // |a| 2^(t - e) < 1/2: rounds to 0
-  // 64-bit limbs S[j] (S[0] = 0, S[j] = limb j - 1; 0 outside, with no
-  // read), all in flight at once: lq - 2 .. lq + W32/2 cover the round bit
-  // (limb lq or lq - 1), the first sticky limbs and the words ws .. ws + W32
-  // of the magnitude
-  auto S = [&](int j) -> uint64_t {
-    return (unsigned)(j - 1) < (unsigned)nl ? __ldg(limbs + (int64_t)(j - 1) * ps + off) : 0ull;
-  };
+  // 64-bit limbs S[j] (S[0] = 0, S[j] = limb j - 1; 0 outside), all in flight
+  // at once: lq - 2 .. lq + W32/2 cover the round bit (limb lq or lq - 1), the
+  // first sticky limbs and the words ws .. ws + W32 of the magnitude
+  auto S = [&](int j) -> uint64_t { return limb(j - 1); };
   const int ws = B >> 5, bs = B & 31, lq = ws >> 1;
   const bool odd = ws & 1;
   constexpr int NLM = W32 / 2 + 3;
@@ -153,187 +149,80 @@ __device__ __forceinline__ void element_words(const uint64_t* __restrict__ limbs
   const uint32_t rb = (uint32_t)(srb >> (rbpos & 63)) & 1u;
   uint64_t sticky = (srb & ((1ull << (rbpos & 63)) - 1ull)) | (rb_hi ? lm[1] : 0ull) | lm[0];
   for (int j = lq - 3; j >= 1 && !sticky; --j) sticky |= S(j);
-  uint32_t c = rb & ((sticky != 0ull) | (wd[0] & 1u));
+  uint64_t y = rb & ((sticky != 0ull) | (wd[0] & 1u));
 #pragma unroll
   for (int w = 0; w < W32; ++w) {                 // |a_hat| <= 2^t fits the W32 words
-    const uint32_t x = wd[w] + c;
-    c = (c && x == 0u) ? 1u : 0u;
-    wd[w] = x;
+    y = (uint64_t)wd[w] + (y >> (w ? 32 : 0));
+    wd[w] = (uint32_t)y;
   }
 }
 
-// Elements per thread of the CUDA-core residue kernel: four while their
-// words fit in registers, else two.
-__host__ __device__ constexpr int residue_ept(int w32) { return w32 <= 10 ? 4 : 2; }
-
-// Centered residue of s |a_hat| mod m from a = sum of the byte products
-// (a == |a_hat| mod m, a < 2^23), in fp32: f = s a exactly; q = f / m rounded
-// to nearest (the 1.5 2^23 addend rounds; q may be off by one because 1/m is
-// rounded), r = f - q m exactly (an fma of integers below 2^24), and one
-// step in each direction brings r into (-m/2, m/2] (ties: +m/2).  The result
-// is an exact small integer; + 0 turns a -0 into +0.
-__device__ __forceinline__ float centered_f32(uint32_t a, bool neg, float mf, float rcp, float hm) {
-  float f = __uint_as_float(a | 0x4B000000u) - 8388608.0f;
-  if (neg) f = -f;
-  const float q = fmaf(f, rcp, 12582912.0f) - 12582912.0f;
-  float r = fmaf(-q, mf, f);
-  r = r > hm ? r - mf : r;
-  r = r <= -hm ? r + mf : r;
-  return r + 0.0f;
-}
+// A block of the residue kernels covers 8 lines x 32 residue_ept k: four where
+// k_residue_frag takes the integers (up to 72 bytes), two beyond (k_residue).
+constexpr int kFragW32 = 18;
+__host__ __device__ constexpr int residue_ept(int w32) { return w32 <= kFragW32 ? 4 : 2; }
 
 // Residues of EPT elements over all L moduli from their first NW words, and
 // the plane writes.  The table row of modulus l holds the packed low bytes of
 // 2^(8 b) mod m_l in words [0, W32) and the high bytes in words [W32, 2 W32).
-// s_mc[l] = {m, floor(2^32 / m), 1/m (fp32 bits), m/2 (fp32 bits)}.  Byte
-// sums stay below 4 NW 255^2 < 2^23 for NW <= 32, so their reduction is done
-// in fp32 there (Barrett beyond, with lo + 256 hi < 2^32 for two-limb moduli).
+// s_mc[l] = {m, floor(2^32 / m)}; lo + 256 hi < 2^32 for two-limb moduli.
 template <int NW, int W32, int EPT>
 __device__ __forceinline__ void residue_planes(const uint32_t (&w)[EPT][W32], const bool (&ng)[EPT],
-                                               const uint32_t* s_t8, const uint4* s_mc, int L, int L1,
+                                               const uint32_t* s_t8, const uint2* s_mc, int L, int L1,
                                                uint16_t* dst, int64_t plane_stride, int nk) {
-  static_assert(EPT == 2 || EPT == 4, "two or four elements per thread");
+  static_assert(EPT == 2, "two elements per thread");
   constexpr int RS = 2 * W32;
-  // per element: s a = fma(s, 2^23 + a, -s 2^23) exactly, +0 for a = 0
-  float sg[EPT], sb[EPT];
-#pragma unroll
-  for (int e = 0; e < EPT; ++e) {
-    sg[e] = ng[e] ? -1.f : 1.f;
-    sb[e] = ng[e] ? 8388608.f : -8388608.f;
-  }
-  // one plane of the EPT elements: one vector store when all are in range;
-  // bits[e] holds the value's bf16 bits in its high half (an exact fp32), two
-  // of them packed by one byte permutation
+  // one plane of the EPT elements: one vector store when both are in range
   auto put = [&](const uint32_t (&bits)[EPT]) {
     if (nk == EPT) {
-      if (EPT == 4) {
-        st_plane4(dst, make_uint2(__byte_perm(bits[0], bits[1], 0x7632), __byte_perm(bits[2], bits[3], 0x7632)));
-      } else {
-        st_plane2(dst, __byte_perm(bits[0], bits[1], 0x7632));
-      }
+      st_plane2(dst, bits[0] | bits[1] << 16);
     } else {
-#pragma unroll
-      for (int e = 0; e < EPT; ++e)
-        if (e < nk) st_plane(dst + e, bits[e] >> 16);
+      st_plane(dst, bits[0]);
     }
     dst += plane_stride;
   };
-  for (int l = 0; l < L; ++l) {
-    const uint4 mcv = s_mc[l];
-    const uint32_t* tw = s_t8 + l * RS;
+  auto sums = [&](const uint32_t* tw, uint32_t (&a)[EPT]) {
     const uint2* tl = reinterpret_cast<const uint2*>(tw);
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) a[e] = 0u;
+#pragma unroll
+    for (int q = 0; q < NW / 2; ++q) {
+      const uint2 t2 = tl[q];
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) {
+        a[e] = __dp4a(w[e][2 * q], t2.x, a[e]);
+        a[e] = __dp4a(w[e][2 * q + 1], t2.y, a[e]);
+      }
+    }
+    if (NW & 1) {
+      const uint32_t tx = tw[NW - 1];
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) a[e] = __dp4a(w[e][NW - 1], tx, a[e]);
+    }
+  };
+  for (int l = 0; l < L; ++l) {
+    const uint2 mc = s_mc[l];
+    uint32_t a[EPT];
+    sums(s_t8 + l * RS, a);
     if (l < L1) {
-      uint32_t a[EPT];
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) a[e] = 0u;
-#pragma unroll
-      for (int q = 0; q < NW / 2; ++q) {
-        const uint2 t2 = tl[q];
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          a[e] = __dp4a(w[e][2 * q], t2.x, a[e]);
-          a[e] = __dp4a(w[e][2 * q + 1], t2.y, a[e]);
-        }
-      }
-      if (NW & 1) {
-        const uint32_t tx = tw[NW - 1];
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) a[e] = __dp4a(w[e][NW - 1], tx, a[e]);
-      }
       uint32_t bits[EPT];
-      if constexpr (NW <= 32) {                             // a < 4 NW 255^2 < 2^23: fp32 reduction
-        const float mf = (float)mcv.x, rcp = __uint_as_float(mcv.z), hm = __uint_as_float(mcv.w);
-        if (mcv.x & 1u) {
-          // odd m: a <= 4 NW 255 250 < 0.973 2^23, so |a rcp - a/m| <=
-          // a 2^-24 (1 + 2^-29) / m < 1/(2m), while a/m is at least 1/(2m)
-          // from every half-integer: the rounded quotient is exact and
-          // r = s a - q m is the centered residue, with no correction step
-          // (an exact zero is +0: x - x and +0 - 0 m round to +0)
 #pragma unroll
-          for (int e = 0; e < EPT; ++e) {
-            const float f = fmaf(sg[e], __uint_as_float(a[e] | 0x4B000000u), sb[e]);
-            const float q = fmaf(f, rcp, 12582912.0f) - 12582912.0f;
-            bits[e] = __float_as_uint(fmaf(-q, mf, f));
-          }
-        } else {                                            // m = 128: ties need the correction
-#pragma unroll
-          for (int e = 0; e < EPT; ++e) bits[e] = __float_as_uint(centered_f32(a[e], ng[e], mf, rcp, hm));
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) bits[e] = bf16_bits(centered(barrett32(a[e], mcv.x, mcv.y), mcv.x, ng[e])) << 16;
-      }
+      for (int e = 0; e < EPT; ++e) bits[e] = bf16_bits(centered(barrett32(a[e], mc.x, mc.y), mc.x, ng[e]));
       put(bits);                                            // plane l
     } else {
-      // low and high table bytes: x = s_lo + 256 s_hi < 2^32
-      uint32_t lo[EPT], hi[EPT];
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) lo[e] = hi[e] = 0u;
-      const uint2* th = tl + W32 / 2;
-#pragma unroll
-      for (int q = 0; q < NW / 2; ++q) {
-        const uint2 t2 = tl[q];
-        const uint2 u2 = th[q];
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          lo[e] = __dp4a(w[e][2 * q], t2.x, lo[e]);
-          lo[e] = __dp4a(w[e][2 * q + 1], t2.y, lo[e]);
-          hi[e] = __dp4a(w[e][2 * q], u2.x, hi[e]);
-          hi[e] = __dp4a(w[e][2 * q + 1], u2.y, hi[e]);
-        }
-      }
-      if (NW & 1) {
-        const uint32_t tx = tw[NW - 1], ux = tw[W32 + NW - 1];
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          lo[e] = __dp4a(w[e][NW - 1], tx, lo[e]);
-          hi[e] = __dp4a(w[e][NW - 1], ux, hi[e]);
-        }
-      }
       // balanced base-128 split: r = r0 + 128 r1 with r0 = cen(r mod 128);
       // planes L1 + 3 (l - L1) + {0, 1, 2} = r0, r1, r0 + r1
-      uint32_t b0[EPT], b1[EPT], b2[EPT];
-      if constexpr (NW <= 32) {
-        // fp32, exact (m odd): lo <= 4 NW 255^2 and hi < lo are below
-        // 2^23 / (1 + 2^-29), so their rounded quotients are exact and give
-        // centered residues; y = r_lo + 256 r_hi has |y| < 2^21, reduced
-        // exactly the same way; then the split with a round-to-nearest
-        // quotient by 128 (a tie leaves r0 = -64, moved to +64)
-        // Up to 24 words lo <= 24 4 255^2 and 256 |r_hi| <= 256 8095 keep
-        // y = s lo + 256 r_hi below 2^23 / (1 + 2^-29): lo needs no reduction
-        // of its own.
-        const float mf = (float)mcv.x, rcp = __uint_as_float(mcv.z);
+      uint32_t hi[EPT], b0[EPT], b1[EPT], b2[EPT];
+      sums(s_t8 + l * RS + W32, hi);
 #pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          const float fl = fmaf(sg[e], __uint_as_float(lo[e] | 0x4B000000u), sb[e]);
-          const float fh = fmaf(sg[e], __uint_as_float(hi[e] | 0x4B000000u), sb[e]);
-          const float qh = fmaf(fh, rcp, 12582912.0f) - 12582912.0f;
-          float yl = fl;
-          if constexpr (NW > 24) {
-            const float ql = fmaf(fl, rcp, 12582912.0f) - 12582912.0f;
-            yl = fmaf(-ql, mf, fl);
-          }
-          const float y = fmaf(256.f, fmaf(-qh, mf, fh), yl);
-          const float q = fmaf(y, rcp, 12582912.0f) - 12582912.0f;
-          const float x = fmaf(-q, mf, y);
-          float r1 = fmaf(x, 0.0078125f, 12582912.0f) - 12582912.0f;
-          float r0 = fmaf(-128.f, r1, x);
-          if (r0 <= -64.f) { r0 += 128.f; r1 -= 1.f; }
-          b0[e] = __float_as_uint(r0);
-          b1[e] = __float_as_uint(r1);
-          b2[e] = __float_as_uint(r0 + r1);
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          const int x = centered(barrett32(lo[e] + (hi[e] << 8), mcv.x, mcv.y), mcv.x, ng[e]);
-          const int y = x & 127;
-          const int r0 = y > 64 ? y - 128 : y;
-          const int r1 = (x - r0) >> 7;
-          b0[e] = bf16_bits(r0) << 16;
-          b1[e] = bf16_bits(r1) << 16;
-          b2[e] = bf16_bits(r0 + r1) << 16;
-        }
+      for (int e = 0; e < EPT; ++e) {
+        const int x = centered(barrett32(a[e] + (hi[e] << 8), mc.x, mc.y), mc.x, ng[e]);
+        const int y = x & 127;
+        const int r0 = y > 64 ? y - 128 : y;
+        const int r1 = (x - r0) >> 7;
+        b0[e] = bf16_bits(r0);
+        b1[e] = bf16_bits(r1);
+        b2[e] = bf16_bits(r0 + r1);
       }
       put(b0);
       put(b1);
@@ -355,12 +244,12 @@ __global__ void __launch_bounds__(256) k_residue(DevTables T, const int4* __rest
   constexpr int W32 = W16 / 2;
   constexpr int EPT = residue_ept(W32);
   constexpr int RS = 2 * W32;                          // table row stride (words)
-  extern __shared__ __align__(16) uint32_t s_t8[];     // [L][RS] packed bytes, then [L] x {m, mu, 1/m, m/2}
+  extern __shared__ __align__(16) uint32_t s_t8[];     // [L][RS] packed bytes, then [L] x {m, mu}
   const int4 b = blk[blockIdx.x];
   const ProbDev& P = T.probs[b.x];
   const int side = b.y;
   const int L = P.L, L1 = P.L1;
-  uint4* s_mc = reinterpret_cast<uint4*>(s_t8 + L * RS);
+  uint2* s_mc = reinterpret_cast<uint2*>(s_t8 + L * RS);
   for (int i = threadIdx.y * 32 + threadIdx.x; i < L * RS; i += 256) {
     const int l = i / RS, d = i - l * RS;         // low bytes [0, W32), high bytes [W32, 2 W32)
     const int src = d < W32 ? d : (T.w16max >> 1) + (d - W32);
@@ -368,7 +257,7 @@ __global__ void __launch_bounds__(256) k_residue(DevTables T, const int4* __rest
   }
   for (int l = threadIdx.y * 32 + threadIdx.x; l < L; l += 256) {
     const ModConst mc = T.mods[l];
-    s_mc[l] = make_uint4(mc.m, mc.mu, __float_as_uint(mc.rcp), __float_as_uint(0.5f * (float)mc.m));
+    s_mc[l] = make_uint2(mc.m, mc.mu);
   }
   __syncthreads();
   const int R = side ? P.N : P.M;
@@ -393,7 +282,9 @@ __global__ void __launch_bounds__(256) k_residue(DevTables T, const int4* __rest
     const int64_t off = off0 + e * stride_k;
     ng[e] = false;
     if (e < nk && __ldg(limbs + (int64_t)(nl - 1) * ps + off) != 0ull) {
-      element_words<W32>(limbs, ps, off, nl, __ldg(exps + off), e_line, P.t, w[e]);
+      element_words<W32>([&](int j) -> uint64_t {
+        return (unsigned)j < (unsigned)nl ? __ldg(limbs + (int64_t)j * ps + off) : 0ull;
+      }, nl, __ldg(exps + off), e_line, P.t, w[e]);
       ng[e] = __ldg(signs + off) != 0;
     } else {
 #pragma unroll
@@ -409,6 +300,299 @@ __global__ void __launch_bounds__(256) k_residue(DevTables T, const int4* __rest
     residue_planes<W32 - 1, W32, EPT>(w, ng, s_t8, s_mc, L, L1, dst, plane_stride, nk);
   else
     residue_planes<W32, W32, EPT>(w, ng, s_t8, s_mc, L, L1, dst, plane_stride, nk);
+}
+
+// The four bytes b_i of x times the element's sign s as f16 pairs
+// {s b0, s b1}, {s b2, s b3} (low half first): the byte permute makes the
+// pair {1024 + b0, 1024 + b1} (each byte under the f16 exponent bits of 2^10,
+// where the mantissa's unit is 1), and one packed fma with s2 = {s, s} and
+// c2 = {-1024 s, -1024 s} leaves s b_i exactly (every value involved is an
+// integer below 2^11; +0 for b_i = 0).
+__device__ __forceinline__ void signed_f16_bytes(uint32_t x, uint32_t s2, uint32_t c2, uint32_t& c01, uint32_t& c23) {
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(c01) : "r"(__byte_perm(x, 0x64646464u, 0x5140)), "r"(s2), "r"(c2));
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(c23) : "r"(__byte_perm(x, 0x64646464u, 0x7362)), "r"(s2), "r"(c2));
+}
+
+// ---------------------------------------------------------------------------
+// Residues of integers of up to 72 bytes, in registers: the byte sums
+// Y[l][e] = sum_b T[l][b] s_e beta_b (T: the low or high bytes of 2^(8 b) mod m_l)
+// as warp-level matrix products of f16 bytes with fp32 sums, exact (products below
+// 2^16, sums below 72 255^2 < 2^23), with the moduli as rows and 32 elements
+// (consecutive k of a line) as columns.
+//
+// A block takes 8 lines x 128 k in four steps of 2 lines x 128 k: each thread
+// integerizes one element into shared words, then each warp takes 32 k of a line.
+// The K order within 16 bytes is permuted on both operands so that thread t of a
+// group of four holds word 4 s + t whole, and the columns of the four products of a
+// tile so that it gets the elements 8 t .. 8 t + 7: its two bf16 planes (two
+// moduli), or the three of a two-limb modulus (low bytes in rows 0-7, high bytes in
+// rows 8-15), leave as 16-byte stores, no exchange between.  The sums are reduced
+// two elements per packed fp32 instruction.
+//
+// What bounds it: instruction issue up to 16 bytes (integerizing is half of it), the
+// latency of the elements' reads at 24 (to 36 bytes) and 16 warps (to 72) per SM
+// beside that, and the plane stores, 2.4 GB at 1531 x 1093 x 1777 with p = 512.
+// Those stores are why a step is long in k: a warp writes 64 bytes of a plane's
+// line, and with a line per warp (8 lines x 32 k) the other halves of the lines of
+// L2 came so much later that p = 512 took 1.26 ms where the pitch is not a multiple
+// of 128 bytes, and 0.61 where it is (here 0.63 and 0.59; 4 lines x 64 k 0.70, at
+// half the sectors per read on side B).  An element's first reads go out a step
+// ahead (without: 1.06 for 1.23 ms at 2048^3 p = 512).
+// Against the dp4a form that this replaces (four byte products per instruction,
+// which the integer pipe takes at a part of the issue rate), ms: 8192^3 p = 53 2.72
+// and 2.21, 2048^3 p = 113 0.29 and 0.25, 1024^3 p = 256 0.180 and 0.130, 2048^3
+// p = 512 1.86 and 1.03, 64 ragged products 6.43 and 4.06.  Against the byte GEMMs
+// with TMEM accumulators (k_residue_mm): 0.27 and 9.8 ms at p = 256 and 53, whose
+// tiles cost more in hand-overs than these few products.
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int frag_steps(int w32) { return (w32 + 3) / 4; }               // K steps of 16 bytes
+__host__ __device__ constexpr int frag_pitch(int w32) { return 4 * (frag_steps(w32) | 1); }   // words per element
+__host__ __device__ constexpr int frag_tiles(int L, int L1) { return (L1 + 15) / 16 + (L - L1 + 7) / 8; }
+__host__ __device__ constexpr int frag_smem(int w32, int tiles) {
+  return tiles * (frag_steps(w32) * 512 + 16 * 8) + 2 * 256 * (frag_pitch(w32) + 1) * 4;
+}
+
+// Two fp32 values in a register pair; a packed instruction rounds each as the
+// scalar one does.
+struct F32x2 { uint64_t v; };
+__device__ __forceinline__ F32x2 f2_pack(float lo, float hi) {
+  F32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(F32x2 x, uint32_t& lo, uint32_t& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(x.v));
+}
+// the bf16 pair of two values exact in bf16
+__device__ __forceinline__ uint32_t f2_bf16(F32x2 x) {
+  uint32_t lo, hi;
+  f2_unpack(x, lo, hi);
+  return __byte_perm(lo, hi, 0x7632);
+}
+__device__ __forceinline__ F32x2 f2_fma(F32x2 a, F32x2 b, F32x2 c) {
+  F32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 f2_add(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+// x y rounded to the nearest integer (|x y| < 2^22)
+__device__ __forceinline__ F32x2 f2_nearest(F32x2 x, F32x2 y) {
+  return f2_add(f2_fma(x, y, f2_pack(12582912.0f, 12582912.0f)), f2_pack(-12582912.0f, -12582912.0f));
+}
+
+// The same words for a significand of one limb and sh <= 63 (t <= 127).
+template <int N>
+__device__ __forceinline__ void words_of_one(uint64_t sig, int sh, uint32_t (&wd)[N]) {
+  uint64_t lo = 0ull, hi = 0ull;
+  if (sh >= 0) {
+    lo = sig << sh;
+    hi = sig >> 1 >> (63 - sh);
+  } else if (sh >= -64) {
+    const uint64_t half = 1ull << 63, rem = sh == -64 ? sig : sig << (64 + sh);   // the bits below
+    lo = sig >> 1 >> (-1 - sh);
+    lo += (rem > half || (rem == half && (lo & 1ull))) ? 1ull : 0ull;
+  }
+  wd[0] = (uint32_t)lo;
+  wd[1] = (uint32_t)(lo >> 32);
+  wd[2] = (uint32_t)hi;
+  wd[3] = (uint32_t)(hi >> 32);
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+template <int W16>
+__global__ void __launch_bounds__(256, W16 > 20 ? 2 : W16 > 12 ? 3 : 4) k_residue_frag(DevTables T, const int4* __restrict__ blk) {
+  constexpr int W32 = W16 / 2, KS = frag_steps(W32), WS = frag_pitch(W32);
+  extern __shared__ __align__(16) uint32_t s_dyn[];
+  __shared__ int s_even;
+  const int4 b = blk[blockIdx.x];
+  const ProbDev& P = T.probs[b.x];
+  const int side = b.y, L = P.L, L1 = P.L1;
+  const int nt1 = (L1 + 15) / 16, ntile = frag_tiles(L, L1);
+  uint4* s_tab = reinterpret_cast<uint4*>(s_dyn);                          // [tile][KS][32] fragments
+  float2* s_mc = reinterpret_cast<float2*>(s_tab + ntile * KS * 32);       // [tile][16] {1/m, -m} of the row
+  uint32_t* s_words = reinterpret_cast<uint32_t*>(s_mc + 16 * ntile);      // [2][256][WS]
+  uint32_t* s_sign = s_words + 2 * 256 * WS;                               // [2][256] the sign as an f16 pair
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) s_even = -1;
+  __syncthreads();
+  // modulus of row r of tile j (-1: none); rows 8-15 of a two-limb tile: the high bytes
+  auto row_mod = [&](int j, int r) {
+    const int l = j < nt1 ? 16 * j + r : L1 + 8 * (j - nt1) + (r & 7);
+    return l < (j < nt1 ? L1 : L) ? l : -1;
+  };
+  const int hw = T.w16max >> 1;
+#pragma unroll 4
+  for (int i = tid; i < ntile * KS * 32; i += 256) {
+    const int j = i / (KS * 32), st = (i >> 5) % KS, g = (i >> 2) & 7, w = 4 * st + (i & 3);
+    auto word = [&](int r) -> uint32_t {
+      const int l = row_mod(j, r);
+      return l >= 0 && w < hw ? __ldg(T.t16 + (int64_t)l * T.w16max + (j >= nt1 && r >= 8 ? hw : 0) + w) : 0u;
+    };
+    const uint32_t x = word(g), y = word(g + 8);
+    s_tab[i] = make_uint4(f16_byte_pair(x, 0x5140), f16_byte_pair(y, 0x5140), f16_byte_pair(x, 0x7362),
+                          f16_byte_pair(y, 0x7362));
+  }
+  for (int i = tid; i < 16 * ntile; i += 256) {
+    const int l = row_mod(i >> 4, i & 15);
+    const ModConst mc = T.mods[max(l, 0)];
+    s_mc[i] = make_float2(mc.rcp, -(float)mc.m);
+    if (l >= 0 && (mc.m & 1u) == 0u) s_even = l;
+  }
+
+  const int R = side ? P.N : P.M, K = P.K, nl = P.nl;
+  const uint64_t* limbs = side ? P.b_limbs : P.a_limbs;
+  const int32_t* exps = side ? P.b_exp : P.a_exp;
+  const int8_t* signs = side ? P.b_sign : P.a_sign;
+  const int64_t ps = side ? P.b_ps : P.a_ps;
+  // this thread's element of a step: line ln of two, k offset kk (memory order), its
+  // slot among the words, and the run of 32 k that its warp reduces
+  const int ln = side ? tid & 1 : tid >> 7, kk = side ? tid >> 1 : tid & 127;
+  const int slot = 128 * ln + (kk & ~31) + 8 * ((kk >> 1) & 3) + 2 * ((kk >> 3) & 3) + (kk & 1);
+  const int wl = warp >> 2, wk = 32 * (warp & 3);
+  const int g = lane >> 2, t4 = lane & 3;
+  const int nks = ((P.W16 + 1) / 2 + 3) / 4;
+  const int64_t pstride = (int64_t)R * P.Kp;
+  uint16_t* const planes = side ? P.pb : P.pa;
+  const int64_t ld = side ? P.b_ld : P.a_ld;
+
+  // an element's first reads, one step ahead of its limbs'
+  uint64_t top = 0ull;
+  int ex = 0, e_line = 0;
+  bool neg = false;
+  int64_t off_next = 0;
+  auto first = [&](int st) {
+    const int r = b.z + 2 * st + ln, k = b.w + kk;
+    const bool in = r < R && k < K;
+    off_next = side ? (int64_t)k * ld + r : (int64_t)r * ld + k;
+    top = in ? __ldg(limbs + (int64_t)(nl - 1) * ps + off_next) : 0ull;
+    ex = in ? __ldg(exps + off_next) : 0;
+    neg = in && __ldg(signs + off_next) != 0;
+    e_line = in ? __ldg((side ? P.f : P.e) + r) : 0;
+  };
+  first(0);
+  for (int sub = 0; sub < 4 && b.z + 2 * sub < R; ++sub) {
+    const int64_t off = off_next;
+    uint32_t wd[4 * KS];
+#pragma unroll
+    for (int q = 0; q < 4 * KS; ++q) wd[q] = 0u;
+    if (top != 0ull) {
+      if (W32 == 4 && nl == 1) {
+        words_of_one(top, ex - e_line + P.t - 64, wd);
+      } else {
+        uint32_t w[W32];
+        element_words<W32>([&](int j) -> uint64_t {
+          return (unsigned)j < (unsigned)nl ? __ldg(limbs + (int64_t)j * ps + off) : 0ull;
+        }, nl, ex, e_line, P.t, w);
+#pragma unroll
+        for (int q = 0; q < W32; ++q) wd[q] = w[q];
+      }
+    }
+    const uint32_t sg = neg ? 0xBC00BC00u : 0x3C003C00u;
+    if (sub < 3) first(sub + 1);
+    uint32_t* const sw = s_words + (sub & 1) * 256 * WS;
+    uint32_t* const ss = s_sign + (sub & 1) * 256;
+#pragma unroll
+    for (int q = 0; q < KS; ++q)
+      *reinterpret_cast<uint4*>(sw + slot * WS + 4 * q) = make_uint4(wd[4 * q], wd[4 * q + 1], wd[4 * q + 2], wd[4 * q + 3]);
+    ss[slot] = sg;
+    __syncthreads();                                  // (the other buffer is read before the next one)
+    const int line = b.z + 2 * sub + wl, k0 = b.w + wk;
+    if (line >= R || k0 >= K) continue;
+    uint16_t* const dst = planes + (int64_t)line * P.Kp + k0 + 8 * t4;
+    uint32_t bf[KS][4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int at = 32 * warp + 8 * j + g;
+      const uint32_t s2 = ss[at], c2 = s2 ^ 0xD800D800u;              // {s, s}, {-1024 s, -1024 s}
+#pragma unroll
+      for (int q = 0; q < KS; ++q) signed_f16_bytes(sw[at * WS + 4 * q + t4], s2, c2, bf[q][j][0], bf[q][j][1]);
+    }
+    const bool store = k0 + 8 * t4 < K;
+    const uint4* tab = s_tab + lane;
+    auto sums = [&](float (&c)[4][4]) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[j][i] = 0.f;
+#pragma unroll
+      for (int q = 0; q < KS; ++q) {
+        if (q == 0 || q < nks) {
+          const uint4 a = tab[32 * q];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mma_f16(c[j], a, bf[q][j][0], bf[q][j][1]);
+        }
+      }
+      tab += 32 * KS;
+    };
+    for (int j = 0; j < nt1; ++j) {
+      float c[4][4];
+      sums(c);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        // odd m: |y| <= 72 255 250 < 0.973 2^23, so |y rcp - y/m| <= |y| 2^-24
+        // (1 + 2^-29) / m < 1/(2m), while y/m is at least 1/(2m) from every
+        // half-integer: the rounded quotient is exact and r = y - q m is the
+        // centered residue.  Even m (128, whose reciprocal and quotients are
+        // exact): only a tie can come out as -m/2.
+        const int l = 16 * j + 8 * h + g;
+        const float2 mc = s_mc[l];
+        const F32x2 rcp = f2_pack(mc.x, mc.x), nm = f2_pack(mc.y, mc.y);
+        uint32_t o[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const F32x2 y = f2_pack(c[q][2 * h], c[q][2 * h + 1]);
+          o[q] = f2_bf16(f2_fma(f2_nearest(y, rcp), nm, y));
+        }
+        if (l == s_even) {
+          const uint32_t tie = __float_as_uint(0.5f * mc.y) >> 16;      // -m/2 in bf16
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if ((o[q] & 0xFFFFu) == tie) o[q] ^= 0x8000u;
+            if ((o[q] >> 16) == tie) o[q] ^= 0x80000000u;
+          }
+        }
+        if (store && l < L1) __stcg(reinterpret_cast<uint4*>(dst + l * pstride), make_uint4(o[0], o[1], o[2], o[3]));
+      }
+    }
+    for (int j = nt1; j < ntile; ++j) {
+      float c[4][4];
+      sums(c);
+      // y = lo + 256 cen(hi): |y| <= 72 255^2 + 256 8095 < 2^23 / (1 + 2^-29), reduced
+      // the same way; then x = r0 + 128 r1 with r1 the nearest of (x - 1/2) / 128
+      // (exact, never a tie: r0 in [-63, 64]); planes r0, r1, r0 + r1
+      const int l = L1 + 8 * (j - nt1) + g;
+      const float2 mc = s_mc[16 * j + g];
+      const F32x2 rcp = f2_pack(mc.x, mc.x), nm = f2_pack(mc.y, mc.y);
+      uint32_t o0[4], o1[4], o2[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const F32x2 lo = f2_pack(c[q][0], c[q][1]), hi = f2_pack(c[q][2], c[q][3]);
+        const F32x2 y = f2_fma(f2_pack(256.f, 256.f), f2_fma(f2_nearest(hi, rcp), nm, hi), lo);
+        const F32x2 x = f2_fma(f2_nearest(y, rcp), nm, y);
+        const F32x2 r1 = f2_nearest(f2_add(x, f2_pack(-0.5f, -0.5f)), f2_pack(0.0078125f, 0.0078125f));
+        const F32x2 r0 = f2_fma(f2_pack(-128.f, -128.f), r1, x);
+        o0[q] = f2_bf16(r0);
+        o1[q] = f2_bf16(r1);
+        o2[q] = f2_bf16(f2_add(r0, r1));
+      }
+      if (store && l < L) {
+        uint16_t* d = dst + (L1 + 3 * (int64_t)(l - L1)) * pstride;
+        __stcg(reinterpret_cast<uint4*>(d), make_uint4(o0[0], o0[1], o0[2], o0[3]));
+        __stcg(reinterpret_cast<uint4*>(d + pstride), make_uint4(o1[0], o1[1], o1[2], o1[3]));
+        __stcg(reinterpret_cast<uint4*>(d + 2 * pstride), make_uint4(o2[0], o2[1], o2[2], o2[3]));
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -726,17 +910,6 @@ struct RmLayout {
     if (total < 116u * 1024u) total = 116u * 1024u;          // one CTA per SM: all 512 TMEM columns
   }
 };
-
-// The four bytes b_i of x times the element's sign s as f16 pairs
-// {s b0, s b1}, {s b2, s b3} (low half first): the byte permute makes the
-// pair {1024 + b0, 1024 + b1} (each byte under the f16 exponent bits of 2^10,
-// where the mantissa's unit is 1), and one packed fma with s2 = {s, s} and
-// c2 = {-1024 s, -1024 s} leaves s b_i exactly (every value involved is an
-// integer below 2^11; +0 for b_i = 0).
-__device__ __forceinline__ void signed_f16_bytes(uint32_t x, uint32_t s2, uint32_t c2, uint32_t& c01, uint32_t& c23) {
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(c01) : "r"(__byte_perm(x, 0x64646464u, 0x5140)), "r"(s2), "r"(c2));
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(c23) : "r"(__byte_perm(x, 0x64646464u, 0x7362)), "r"(s2), "r"(c2));
-}
 
 // Centered residue of an exact fp32 integer y (|y| < 2^24): y - q m with q the
 // round-to-nearest of y / m (the 1.5 2^23 addend rounds; q may be off by one
@@ -1209,12 +1382,23 @@ int residue_class_for(int w16) {
   return -1;
 }
 int residue_class_w16(int cls) { return kResidueW16[cls]; }
+int residue_class_smem(int cls, int lmax, int tiles) {
+  const int w16 = kResidueW16[cls];
+  return w16 / 2 <= kFragW32 ? frag_smem(w16 / 2, tiles) : lmax * (w16 + 2) * 4;
+}
+int residue_tiles(int L, int L1) { return frag_tiles(L, L1); }
 int residue_class_ept(int cls) { return residue_ept(kResidueW16[cls] / 2); }
 
 cudaError_t launch_scan(const DevTables& t, int /*count*/, const int32_t* blk_rows,
                         const int32_t* blk_cols, int nblk_rows, int nblk_cols, cudaStream_t s) {
   if (nblk_rows) k_scan<<<nblk_rows, 256, 0, s>>>(t, reinterpret_cast<const int4*>(blk_rows));
   if (nblk_cols) k_scan<<<nblk_cols, 256, 0, s>>>(t, reinterpret_cast<const int4*>(blk_cols));
+  return cudaGetLastError();
+}
+
+template <int W16>
+static cudaError_t launch_frag(const DevTables& t, const int4* blk, int nblk, int smem, cudaStream_t s) {
+  k_residue_frag<W16><<<nblk, 256, smem, s>>>(t, blk);
   return cudaGetLastError();
 }
 
@@ -1230,10 +1414,10 @@ static cudaError_t launch_res_w(const DevTables& t, const int4* blk, int nblk, i
 cudaError_t init_prep_attributes() {
   const int mx = 200 * 1024;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue<20>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue<36>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue_frag<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue_frag<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue_frag<20>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue_frag<36>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue<68>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue<132>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_residue_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
@@ -1246,10 +1430,10 @@ cudaError_t launch_residues(const DevTables& t, int cls, const int32_t* blk_list
   const int4* blk = reinterpret_cast<const int4*>(blk_list);
   if (nblk == 0) return cudaSuccess;
   switch (cls) {
-    case 0: return launch_res_w<8>(t, blk, nblk, smem_bytes, s);
-    case 1: return launch_res_w<12>(t, blk, nblk, smem_bytes, s);
-    case 2: return launch_res_w<20>(t, blk, nblk, smem_bytes, s);
-    case 3: return launch_res_w<36>(t, blk, nblk, smem_bytes, s);
+    case 0: return launch_frag<8>(t, blk, nblk, smem_bytes, s);
+    case 1: return launch_frag<12>(t, blk, nblk, smem_bytes, s);
+    case 2: return launch_frag<20>(t, blk, nblk, smem_bytes, s);
+    case 3: return launch_frag<36>(t, blk, nblk, smem_bytes, s);
     case 4: return launch_res_w<68>(t, blk, nblk, smem_bytes, s);
     case 5: return launch_res_w<132>(t, blk, nblk, smem_bytes, s);
   }
