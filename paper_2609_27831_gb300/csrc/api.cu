@@ -354,6 +354,38 @@ static int modulus_prefix(int64_t inner, int t, int force_L, Big* P) {
   return big_cmp(*P, bound) <= 0 ? -1 : L;
 }
 
+// f16 bits of an integer |x| <= 2048 (exact)
+static uint16_t f16_int(int x) {
+  if (x == 0) return 0;
+  const uint16_t sgn = x < 0 ? 0x8000u : 0u;
+  const uint32_t a = (uint32_t)(x < 0 ? -x : x);
+  int e = 0;
+  while ((a >> (e + 1)) != 0u) ++e;           // a in [2^e, 2^(e+1))
+  return (uint16_t)(sgn | (uint32_t)(e + 15) << 10 | ((a << (10 - e)) & 0x3FFu));
+}
+
+// The operand fragments of k_crt_frag after the digit tables `words` of a modulus
+// set: column c of tile j is byte 2 (j % 2) + c % 2 of digit c / 2 + 4 (j / 2) of M_l;
+// the last digit's columns are the bytes of floor(2^32 / m_l).
+static void append_crt_fragments(const CrtHost& c, std::vector<uint32_t>& words) {
+  const int L = c.L, DS = c.DS;
+  const auto& mlist = modulus_list();
+  words.resize(crt_frag_offset(L, DS), 0u);
+  auto value = [&](int l, int digit, int byte) -> uint32_t {
+    if (l >= L) return 0;
+    const uint32_t w = digit < DS - 1 ? c.words[3 * DS + L + (size_t)l * DS + digit]
+                                      : (uint32_t)((1ull << 32) / (uint64_t)mlist[l]);
+    return f16_int((int)((w >> (8 * byte)) & 255u));
+  };
+  for (int s = 0; 16 * s < L; ++s)
+    for (int j = 0; j < DS / 2; ++j)
+      for (int lane = 0; lane < 32; ++lane) {
+        const int g = lane >> 2, l = 16 * s + 2 * (lane & 3), digit = (g >> 1) + 4 * (j >> 1), byte = 2 * (j & 1) + (g & 1);
+        for (int h = 0; h < 16; h += 8)
+          words.push_back(value(l + h, digit, byte) | value(l + h + 1, digit, byte) << 16);
+      }
+}
+
 // Tensor-core residue table [rows][kpad] (f16 bits) of the moduli
 // l0 .. l0 + L - 1 of the list (L1 of them one-limb): row l (one-limb) =
 // cen(2^(8 b) mod m), rows L1 + 2 (l - L1) + {0, 1} (two-limb) = the balanced
@@ -367,14 +399,7 @@ static int res_table_key(ozaki2_plan_s* pl, int l0, int L, int L1, int nb, int k
   ResTable rt;
   rt.l0 = l0; rt.L = L; rt.kpad = kpad; rt.npad = npad; rt.rows = rows;
   rt.bits.assign((size_t)rows * kpad, 0);
-  auto bf = [](int x) -> uint16_t {   // f16 bits of an integer |x| <= 2048 (exact)
-    if (x == 0) return 0;
-    const uint16_t sgn = x < 0 ? 0x8000u : 0u;
-    const uint32_t a = (uint32_t)(x < 0 ? -x : x);
-    int e = 0;
-    while ((a >> (e + 1)) != 0u) ++e;           // a in [2^e, 2^(e+1))
-    return (uint16_t)(sgn | (uint32_t)(e + 15) << 10 | ((a << (10 - e)) & 0x3FFu));
-  };
+  auto bf = f16_int;
   const auto& mlist = modulus_list();
   for (int l = 0; l < L; ++l) {
     const int m = (int)mlist[l0 + l];
@@ -491,6 +516,8 @@ static int build_problem(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int
     key = (int)pl->crts.size() - 1;
   }
   h.crt_key = key;
+  // (k_crt_frag: bytes of v_l, DS / 4 steps of 16 moduli)
+  if (h.DS <= kCrtFragDigits && (h.L != h.L1 || h.L > 4 * h.DS)) return OZ2_EINTERNAL;
   {
     CrtHost& c = pl->crts[key];
     const int np = (big_bitlen(c.P) + 6) / 7 + 1;
@@ -901,7 +928,9 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
   std::vector<int> key_off(pl->crts.size());
   for (size_t i = 0; i < pl->crts.size(); ++i) {
     key_off[i] = (int)pool.size();
-    pool.insert(pool.end(), pl->crts[i].words.begin(), pl->crts[i].words.end());
+    std::vector<uint32_t> words = pl->crts[i].words;
+    if (pl->crts[i].DS <= kCrtFragDigits) append_crt_fragments(pl->crts[i], words);
+    pool.insert(pool.end(), words.begin(), words.end());
     pool.resize(align_up(pool.size(), 64), 0u);
   }
   d.crt_off.resize(count);

@@ -582,6 +582,143 @@ __global__ void __launch_bounds__(kEpb1) k_crt1(DevTables T, const int4* __restr
 
 
 // ---------------------------------------------------------------------------
+// The same for accumulators of up to 12 digits, whose moduli all have one limb:
+// S = sum_l v_l M_l by bytes of M_l, as warp-level products of f16 values (v_l and
+// bytes below 2^8, fp32 sums below 48 255^2 < 2^22, exact), outputs as rows and
+// bytes as columns.  The top digit column holds the bytes of floor(2^32 / m_l),
+// whose sum gives the quotient estimate (M_l has no digit there).  The columns are
+// permuted so that thread t of a group of four gets the digits t, t + 4, ... of its
+// rows whole; they go through shared memory to the lane that finishes the output.
+// The operand rows come out of the staged v_l by transposing matrix loads; the byte
+// table is read as fragments, laid out by the host.
+// What bounds it: the instruction issue, more than half of it now the comparison,
+// rounding and writing of an output.  Against k_crt1 at 8 and 12 digits (a 64-bit
+// multiply-add per modulus and digit and a table read per four), ms: 8192^2 outputs
+// of p = 53 2.88 and 1.7, 2048^2 of p = 113 0.371 and 0.197.
+// ---------------------------------------------------------------------------
+constexpr int kCfPitch = kEpb1 + 8;                 // v_l row: eight rows meet no bank twice
+constexpr int kCfCol = 36;                          // outputs of a digit row (64-bit), 32 and padding
+
+__device__ __forceinline__ void mma_f16_crt(float (&c)[4], const uint32_t (&a)[4], uint2 b) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+template <int ND>
+__global__ void __launch_bounds__(kEpb1) k_crt_frag(DevTables T, const int4* __restrict__ blk) {
+  constexpr int NT = ND / 2, KMAX = ND / 4;         // column tiles of 8 bytes, steps of 16 moduli
+  __shared__ __align__(16) uint16_t s_v[16 * KMAX * kCfPitch];
+  __shared__ __align__(16) uint64_t s_x[(kEpb1 / 32) * ND * kCfCol];
+  __shared__ uint32_t s_tab[3 * ND];                // negP, negH1, P
+  const int4 b = blk[blockIdx.x];
+  const ProbDev& P = T.probs[b.x];
+  const int64_t MN = (int64_t)P.M * P.N;
+  const int64_t e0 = (int64_t)b.y * kEpb1;
+  const int L = P.L, D = P.D32, ks = (L + 15) / 16;
+  const CrtView cv = crt_view(T.crt_pool, P);
+  const int e = threadIdx.x, warp = e >> 5, lane = e & 31;
+  const int64_t idx = e0 + e;
+  const int ef = idx < MN ? crt_ef(P, idx) : 0;     // early: used by the rounding
+  // v_l as the plane GEMM stored it: 16-byte loads of 8 values, independent loads
+  // first; zeros past L
+  {
+    const int lane8 = e & 15, lrow = e >> 4;
+    const bool full = e0 + kEpb1 <= MN;
+    uint4 w[2 * KMAX];
+#pragma unroll
+    for (int j = 0; j < 2 * KMAX; ++j) {
+      const int l = 8 * j + lrow;
+      w[j] = make_uint4(0u, 0u, 0u, 0u);
+      if (l < L) {
+        const uint16_t* src = P.u + (int64_t)l * P.upitch + e0 + 8 * lane8;
+        if (full) {
+          w[j] = __ldg(reinterpret_cast<const uint4*>(src));
+        } else {
+          uint16_t tmp[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) tmp[q] = (e0 + 8 * lane8 + q < MN) ? src[q] : (uint16_t)0;
+          w[j].x = tmp[0] | ((uint32_t)tmp[1] << 16); w[j].y = tmp[2] | ((uint32_t)tmp[3] << 16);
+          w[j].z = tmp[4] | ((uint32_t)tmp[5] << 16); w[j].w = tmp[6] | ((uint32_t)tmp[7] << 16);
+        }
+      }
+    }
+    for (int i = e; i < ND; i += kEpb1) {
+      s_tab[i] = i < D ? __ldg(cv.negP + i) : ~0u;           // widened to ND digits (crt_finish)
+      s_tab[ND + i] = i < D ? __ldg(cv.negH1 + i) : ~0u;
+      s_tab[2 * ND + i] = i < D ? __ldg(cv.P + i) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < 2 * KMAX; ++j) *reinterpret_cast<uint4*>(s_v + (8 * j + lrow) * kCfPitch + 8 * lane8) = w[j];
+  }
+  uint2 bf[KMAX][NT];
+  const uint2* tab = reinterpret_cast<const uint2*>(crt_frag_table(cv, P)) + lane;
+#pragma unroll
+  for (int s = 0; s < KMAX; ++s)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) bf[s][j] = s < ks ? __ldg(tab + (s * NT + j) * 32) : make_uint2(0u, 0u);
+  __syncthreads();
+
+  uint64_t* const x = s_x + warp * ND * kCfCol;
+  const int g = lane >> 2, t4 = lane & 3;
+  // lanes 8 i + r point at row r of matrix i: moduli 8 (i / 2) + r, outputs 8 (i % 2) ..
+  const uint32_t vaddr =
+      tc::smem_u32(s_v + ((lane >> 4) * 8 + (lane & 7)) * kCfPitch + 32 * warp + 8 * ((lane >> 3) & 1));
+#pragma unroll
+  for (int mt = 0; mt < 2; ++mt) {
+    float c[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c[j][i] = 0.f;
+#pragma unroll
+    for (int s = 0; s < KMAX; ++s) {
+      if (s > 0 && s >= ks) break;
+      uint32_t a[4];
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                   : "r"(vaddr + (uint32_t)(2 * (16 * s * kCfPitch + 16 * mt))));
+#pragma unroll
+      for (int i = 0; i < 4; ++i)                   // an integer below 2^8 as f16: (1024 + v) - 1024
+        asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(a[i]) : "r"(a[i] | 0x64006400u), "r"(0x64006400u));
+#pragma unroll
+      for (int j = 0; j < NT; ++j) mma_f16_crt(c[j], a, bf[s][j]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < ND / 4; ++i) {
+        // four byte sums of a digit: the bits of 2^23 + y are 0x4B000000 + y
+        uint32_t y[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = __float_as_uint(c[2 * i + (q >> 1)][2 * h + (q & 1)] + 8388608.0f);
+        constexpr uint32_t kBias = 0x4B000000u + (0x4B000000u << 8);
+        const uint32_t lo = y[0] + (y[1] << 8) - kBias, hi = y[2] + (y[3] << 8) - kBias;
+        x[(t4 + 4 * i) * kCfCol + 16 * mt + 8 * h + g] = lo + ((uint64_t)hi << 16);
+      }
+  }
+  __syncwarp();
+  uint64_t acc[ND];
+#pragma unroll
+  for (int d = 0; d < ND; ++d) acc[d] = x[d * kCfCol + lane];
+  __syncwarp();                                     // s_x becomes the digits' scratch
+  if (idx >= MN) return;
+  // quotient estimate alpha~ in {alpha - 1, alpha}; R = S + alpha~ (2^(32 D) - P) mod 2^(32 D)
+  const uint64_t alpha = acc[ND - 1] >> 32;
+  acc[ND - 1] = 0ull;
+  uint32_t R[ND];
+  uint64_t cy = 0;
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    const uint64_t z = acc[d] + alpha * s_tab[d] + cy;
+    R[d] = d < D ? (uint32_t)z : 0u;
+    cy = z >> 32;
+  }
+  crt_finish<ND>(P, R, s_tab, reinterpret_cast<uint32_t*>(x), 32, lane, idx, ef, T.status);
+}
+
+// ---------------------------------------------------------------------------
 // CRT column sums on the tensor cores.  With v_l = v0 + 128 v1 (7-bit halves)
 // and M_l = sum_j M_l[j] 128^j (7-bit pieces),
 //   S = sum_l v_l M_l = sum_j 128^j Y_j,   Y_j = sum_l (v0_l M_l[j] + v1_l M_l[j-1]),
@@ -1695,6 +1832,12 @@ cudaError_t crt1_attr() {
 }
 
 template <int ND>
+cudaError_t launch_crt_frag(const DevTables& t, const int4* blk, int nblk, cudaStream_t s) {
+  k_crt_frag<ND><<<nblk, kEpb1, 0, s>>>(t, blk);
+  return cudaGetLastError();
+}
+
+template <int ND>
 cudaError_t launch_crt1_t(const DevTables& t, const int4* blk, int nblk, int lmax, cudaStream_t s) {
   const int smem = lmax * ND * 4 + lmax * 4 + 3 * ND * 4 + ND * kEpb1 * 4 + lmax * kEpb1 * 2 + 16;
   k_crt1<ND><<<nblk, kEpb1, smem, s>>>(t, blk);
@@ -1802,8 +1945,6 @@ cudaError_t init_crt_attributes() {
   cudaError_t e = cudaFuncSetAttribute(k_crt_mm, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_crt_fin_long, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e == cudaSuccess) e = crt1_attr<8>();
-  if (e == cudaSuccess) e = crt1_attr<12>();
   if (e == cudaSuccess) e = crt1_attr<16>();
   if (e == cudaSuccess) e = crt1_attr<20>();
   if (e == cudaSuccess) e = crt1_attr<24>();
@@ -1846,8 +1987,8 @@ cudaError_t launch_crt(const DevTables& t, int cls, const int32_t* blk_list, int
   const int4* blk = reinterpret_cast<const int4*>(blk_list);
   const int smem = lmax * crt_class_elems_per_block(cls) * 2;
   switch (cls) {
-    case 0: return launch_crt1_t<8>(t, blk, nblk, lmax, s);
-    case 1: return launch_crt1_t<12>(t, blk, nblk, lmax, s);
+    case 0: return launch_crt_frag<8>(t, blk, nblk, s);
+    case 1: return launch_crt_frag<12>(t, blk, nblk, s);
     case 2: return launch_crt1_t<16>(t, blk, nblk, lmax, s);
     case 3: return launch_crt1_t<20>(t, blk, nblk, lmax, s);
     case 4: return launch_crt1_t<24>(t, blk, nblk, lmax, s);

@@ -130,6 +130,15 @@ __host__ __device__ inline CrtView crt_view(const uint32_t* pool, const ProbDev&
   return v;
 }
 
+// Accumulators of up to 12 digits (classes 0 and 1, DS of 8 and 12) append the bytes
+// of M_l to their tables as operand fragments of k_crt_frag: [step of 16 moduli]
+// [tile of 8 columns][32 lanes] of two f16 pairs.
+constexpr int kCrtFragDigits = 12;
+__host__ __device__ inline size_t crt_frag_offset(int L, int DS) { return (3 * (size_t)DS + L + (size_t)L * DS + 1) / 2 * 2; }
+__host__ __device__ inline const uint32_t* crt_frag_table(const CrtView& v, const ProbDev& pr) {
+  return v.P + crt_frag_offset(pr.L, pr.DS);
+}
+
 // One (modulus, output tile) work unit of the grouped GEMM.
 struct Unit {
   uint16_t prob;
