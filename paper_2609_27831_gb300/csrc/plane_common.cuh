@@ -5,6 +5,7 @@
 
 #include <cstdint>
 
+#include "f32x2.cuh"
 #include "oz2_internal.h"
 #include "tc_ptx.cuh"
 
@@ -17,22 +18,23 @@ __device__ __forceinline__ uint32_t barrett32(uint32_t x, uint32_t m, uint32_t m
   return r >= m ? r - m : r;
 }
 
-// x: exact integer held in fp32 with |x| < 2^25.  Returns x mod m in [0, m).
-// q = rint(x * rcp) is within 0.52 of x/m, so r = x - q m lies in
-// (-0.52 m, 0.52 m) and is computed exactly by the fma; one correction
-// brings it into [0, m).
-__device__ __forceinline__ uint32_t fmod_small(float x, float mf, float rcp) {
-  const float q = rintf(x * rcp);
-  float r = fmaf(-q, mf, x);
-  r = r < 0.f ? r + mf : r;
-  // exact float -> int of 0 <= r < 2^23 without a conversion instruction
-  return __float_as_uint(r + 8388608.0f) - 0x4B000000u;
-}
-
-// exact int -> float of 0 <= x < 2^23 without a conversion instruction
-__device__ __forceinline__ float small_u2f(uint32_t x) {
-  return __uint_as_float(0x4B000000u + x) - 8388608.0f;
-}
+// The epilogue's reductions, two values per packed fp32 instruction, all on exact
+// integers.  Scalar, with the products in 32-bit Barrett form, they took about 12
+// instructions per value (plane GEMMs so and now, ms: 4096^3 p = 2048 68.3 and 65.6,
+// 1024^3 p = 256 0.141 and 0.138, 64 ragged products 8.68 and 8.49).
+struct EpiMod {
+  F32x2 rcp, nm, h;   // 1/m, -m, -(m - 1) / (2 m)
+  // x mod m, |x| < 2^24: the quotient is within 0.52 of x / m, the result within
+  // 0.52 m of zero
+  __device__ __forceinline__ F32x2 centered(F32x2 x) const { return f2_fma(f2_nearest(x, rcp), nm, x); }
+  // x mod m in [0, m): (x - (m - 1) / 2) / m is 1 / (2 m) or more away from every
+  // half-integer and its nearest integer is floor(x / m); exact while the error of
+  // x / m, 2^-23 |x| / m, stays below that: |x| < 2^22
+  __device__ __forceinline__ F32x2 floored(F32x2 x) const {
+    const F32x2 one = f2_pack(1.f, 1.f);
+    return f2_fma(f2_nearest(f2_fma(x, rcp, h), one), nm, x);
+  }
+};
 
 // One accumulation job: plane `plane` of unit `u` over K chunk `chunk`.
 struct Job {
@@ -131,8 +133,7 @@ static __device__ __noinline__ void dbg_write_back(int32_t* dbg, int plane, int 
 // loads run while the epilogue waits for the slot; the chunk loop then reads
 // no global memory but the optional debug dump).
 struct EpiConst {
-  float mf, rcp;
-  uint32_t m, mu;
+  float mf, rcp, hf;  // m, 1/m, -(m - 1) / (2 m)
   uint32_t mul;       // write-back: the next plane's Karatsuba factor; last job:
                       // kfin M_l^{-1} mod m_l, so that the stored value is the
                       // CRT's v_l = (c mod m_l) M_l^{-1} mod m_l (Sec. 4.4)
@@ -159,8 +160,7 @@ __device__ __forceinline__ EpiConst epi_const(const DevTables& T, const Job& j, 
   EpiConst e;
   e.mf = (float)mc.m;
   e.rcp = mc.rcp;
-  e.m = mc.m;
-  e.mu = mc.mu;
+  e.hf = -0.5f * (e.mf - 1.f) / e.mf;
   e.M = P.M;
   e.N = P.N;
   e.row = row;
@@ -210,22 +210,35 @@ __device__ __forceinline__ void epi_chunk(const Job& j, const EpiConst& e, uint3
                                           int cc, UStage& us) {
   const int col = e.col0 + cc;
   if (e.dbg != nullptr) dbg_plane_sums(e.dbg, j.plane, j.first, e.M, e.N, e.row, col, taddr);
+  const EpiMod md{f2_pack(e.rcp, e.rcp), f2_pack(-e.mf, -e.mf), f2_pack(e.hf, e.hf)};
+  const bool two = e.ell >= e.L1;
+  // a factor below 2^14 in halves of 7 bits (x times a half below 2^22), or whole below 2^8
+  const float f0 = (float)(two ? e.mul & 127u : e.mul), f1 = (float)(e.mul >> 7);
+  const F32x2 m0 = f2_pack(f0, f0), m1 = f2_pack(f1, f1), zero = f2_pack(0.f, 0.f);
+  // x mul as 128 cen(x m1) + x m0, |.| < 2^22
+  auto times = [&](F32x2 x) {
+    return f2_fma(f2_pack(128.f, 128.f), md.centered(f2_fma(x, m1, zero)), f2_fma(x, m0, zero));
+  };
   if (!j.last) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      uint32_t r = fmod_small(__uint_as_float(v[i]), e.mf, e.rcp);
-      if (e.mul != 1u) r = barrett32(r * e.mul, e.m, e.mu);
-      v[i] = __float_as_uint(small_u2f(r));
+    for (int i = 0; i < 32; i += 2) {
+      F32x2 x = md.centered(f2_pack(v[i], v[i + 1]));
+      if (e.mul != 1u) x = md.centered(times(x));            // two-limb moduli
+      f2_unpack(x, v[i], v[i + 1]);
     }
     tc::tmem_st32(taddr, v);
     if (e.dbg != nullptr) dbg_write_back(e.dbg, j.plane, j.u.ell, e.L1, e.M, e.N, e.row, col, taddr);
     return;
   }
+  // v_l in [0, m), two to a word: one-limb |x mul| < 2^16; two-limb once more centered first
+  const F32x2 up = f2_pack(8388608.0f, 8388608.0f);          // the bits of 2^23 + v end in v
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    uint32_t r = fmod_small(__uint_as_float(v[i]), e.mf, e.rcp);
-    if (e.mul != 1u) r = barrett32(r * e.mul, e.m, e.mu);
-    v[i] = r;
+  for (int i = 0; i < 32; i += 2) {
+    F32x2 x = md.centered(f2_pack(v[i], v[i + 1]));
+    if (two) x = md.centered(times(x));
+    else x = f2_fma(x, m0, zero);
+    f2_unpack(f2_add(md.floored(x), up), v[i], v[i + 1]);
+    v[i >> 1] = __byte_perm(v[i], v[i + 1], 0x5410);
   }
   // staged tile: by TMA where u's rows allow it, else row by row
   const int lane = threadIdx.x & 31;
@@ -243,9 +256,8 @@ __device__ __forceinline__ void epi_chunk(const Job& j, const EpiConst& e, uint3
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q)
-    tc::st_shared_v4(buf + (uint32_t)(lane * 64 + 16 * (q ^ ((lane >> 1) & 3))), v[8 * q] | (v[8 * q + 1] << 16),
-                     v[8 * q + 2] | (v[8 * q + 3] << 16), v[8 * q + 4] | (v[8 * q + 5] << 16),
-                     v[8 * q + 6] | (v[8 * q + 7] << 16));
+    tc::st_shared_v4(buf + (uint32_t)(lane * 64 + 16 * (q ^ ((lane >> 1) & 3))), v[4 * q], v[4 * q + 1],
+                     v[4 * q + 2], v[4 * q + 3]);
   ++us.n;
   if (us.map != nullptr) {
     tc::fence_proxy_async_smem();

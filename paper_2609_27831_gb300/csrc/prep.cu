@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "f32x2.cuh"
 #include "oz2_internal.h"
 #include "tc_ptx.cuh"
 
@@ -350,38 +351,6 @@ __host__ __device__ constexpr int frag_pitch(int w32) { return 4 * (frag_steps(w
 __host__ __device__ constexpr int frag_tiles(int L, int L1) { return (L1 + 15) / 16 + (L - L1 + 7) / 8; }
 __host__ __device__ constexpr int frag_smem(int w32, int tiles) {
   return tiles * (frag_steps(w32) * 512 + 16 * 8) + 2 * 256 * (frag_pitch(w32) + 1) * 4;
-}
-
-// Two fp32 values in a register pair; a packed instruction rounds each as the
-// scalar one does.
-struct F32x2 { uint64_t v; };
-__device__ __forceinline__ F32x2 f2_pack(float lo, float hi) {
-  F32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void f2_unpack(F32x2 x, uint32_t& lo, uint32_t& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(x.v));
-}
-// the bf16 pair of two values exact in bf16
-__device__ __forceinline__ uint32_t f2_bf16(F32x2 x) {
-  uint32_t lo, hi;
-  f2_unpack(x, lo, hi);
-  return __byte_perm(lo, hi, 0x7632);
-}
-__device__ __forceinline__ F32x2 f2_fma(F32x2 a, F32x2 b, F32x2 c) {
-  F32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-__device__ __forceinline__ F32x2 f2_add(F32x2 a, F32x2 b) {
-  F32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-// x y rounded to the nearest integer (|x y| < 2^22)
-__device__ __forceinline__ F32x2 f2_nearest(F32x2 x, F32x2 y) {
-  return f2_add(f2_fma(x, y, f2_pack(12582912.0f, 12582912.0f)), f2_pack(-12582912.0f, -12582912.0f));
 }
 
 // The same words for a significand of one limb and sh <= 63 (t <= 127).
