@@ -855,16 +855,21 @@ __global__ void __launch_bounds__(kRtThreads, 2)
 //               t & 1 for tile t: integerize the tile's elements and write
 //               their bytes into A buffer t mod nabuf once the MMAs of tile
 //               t - nabuf are done, so that two tiles are built at once
-//   warps 10-21 three per lane quadrant (sub-groups s = 0..2): the tile's
-//               32-column groups in turn (rotated per tile); a group is all
+//   warps 10-25 four per lane quadrant (sub-groups s = 0..3): the tile's
+//               16-column groups in turn (rotated per tile); a group is all
 //               one-limb, all two-limb pairs (L1 is even) or the one mixed
 //               group: reduce mod m_l (round-to-nearest quotient in fp32, the
 //               sign applied first), split two-limb residues, store the bf16
 //               planes through incremental plane pointers.
+// What bounds it: the epilogue, whose warps work 26 of a tile's 30 thousand cycles at
+// 1024^3 p = 2048 (builders 11 and waits, MMA issue 9).  Three warps per quadrant in
+// 32-column groups took 1.63 ms there (0.80 at p = 1024, 37.0 at 4096^3 p = 2048), four
+// in 32-column groups 1.58, in 16-column ones 1.49 (0.72, 34.6); pairs of planes as
+// 4-byte stores across two lanes took 1.68.
 // Tile list entry: {problem, side, first line, first k}.
 // ---------------------------------------------------------------------------
 constexpr int kRmBuilders = 256;                  // two groups of four warps
-constexpr int kRmEpi = 384;                       // three warps per lane quadrant
+constexpr int kRmEpi = 512;                       // four warps per lane quadrant
 constexpr int kRmThreads = 64 + kRmBuilders + kRmEpi;
 constexpr int kRmMaxStages = 16;
 
@@ -1161,7 +1166,7 @@ __global__ void __launch_bounds__(kRmThreads, 1)
   } else {
     // ------------------------------------------------------------ epilogues
     const int ew = warp - 10;
-    const int sub = ew >> 2;                          // column sub-group 0..2
+    const int sub = ew >> 2;                          // column sub-group 0..3
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
     const uint32_t tlane = tmem + ((uint32_t)(quad * 32) << 16);
@@ -1189,75 +1194,70 @@ __global__ void __launch_bounds__(kRmThreads, 1)
         const uint32_t trow = tlane + (uint32_t)nabuf * acols + (uint32_t)(s * cw);
         const int j0 = c * cw;
         const int ncolp = min(cw, npad - j0);          // columns written by the MMAs
-        // the tile's 32-column groups go round the three sub-groups (rotated
-        // per tile), whatever the chunk width
-        const int gfirst = ((sub - c * (cw >> 5) - tcount) % 3 + 3) % 3;
-        for (int g = 32 * gfirst; g < ncolp; g += 96) {
-          // 16 columns per TMEM load, reduced as two pieces of 8 (a rolled
-          // loop: the epilogue's code stays small next to the builders' in
-          // the instruction cache); pieces hold whole pairs (L1 and every
-          // piece start are even)
-          const int gcols = min(32, ncolp - g);           // 32 or 16
+        // the tile's 16-column groups go round the four sub-groups (rotated
+        // per tile), whatever the chunk width: 16 columns per TMEM load,
+        // reduced as two pieces of 8 (a rolled loop: the epilogue's code stays
+        // small next to the builders' in the instruction cache); pieces hold
+        // whole pairs (L1 and every piece start are even)
 #pragma unroll 1
-          for (int pc2 = 0; pc2 < gcols; pc2 += 16) {
-            uint32_t y16[16];
-            tmem_ld16(trow + (uint32_t)(g + pc2), y16);
-            if (!valid) continue;
+        for (int g = 16 * ((sub - c * (cw >> 4) - tcount) & 3); g < ncolp; g += 64) {
+          uint32_t y16[16];
+          tmem_ld16(trow + (uint32_t)g, y16);
+          if (!valid) continue;
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              const int pc = pc2 + 8 * hh;
-              uint32_t y[8];
+          for (int hh = 0; hh < 2; ++hh) {
+            const int pc = 8 * hh;
+            uint32_t y[8];
 #pragma unroll
-              for (int q = 0; q < 8; ++q) y[q] = y16[8 * hh + q];
-              const int c0 = j0 + g + pc;
-              if (c0 + 8 <= L1) {
-                // 8 one-limb moduli: planes c0 .. c0 + 7
-                uint16_t* dp = dst0 + (int64_t)c0 * pstride;
+            for (int q = 0; q < 8; ++q) y[q] = y16[8 * hh + q];
+            const int c0 = j0 + g + pc;
+            if (c0 + 8 <= L1) {
+              // 8 one-limb moduli: planes c0 .. c0 + 7
+              uint16_t* dp = dst0 + (int64_t)c0 * pstride;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                  const float4 mc = s_mc[c0 + q];
+              for (int q = 0; q < 8; ++q) {
+                const float4 mc = s_mc[c0 + q];
+                const float r = cmod_f32(__uint_as_float(y[q]), mc.x, mc.y, mc.z) + 0.0f;
+                *dp = (uint16_t)(__float_as_uint(r) >> 16);
+                dp += pstride;
+              }
+            } else if (c0 >= L1) {
+              // 4 two-limb pairs: moduli l = L1 + (c0 - L1) / 2 + i, planes L1 + 3 (l - L1) + {0, 1, 2}
+              const int lb = L1 + ((c0 - L1) >> 1);
+              uint16_t* dp = dst0 + (int64_t)(L1 + 3 * (lb - L1)) * pstride;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                if (c0 + 2 * i < ncols) {
+                  const float4 mc = s_mc[lb + i];
+                  // x is +0 for a zero residue; then lo, hi and lo + hi are never -0
+                  const float x = cmod2_f32(y[2 * i], y[2 * i + 1], mc.x, mc.y);
+                  float lo, hi;
+                  split128(x, lo, hi);
+                  dp[0] = (uint16_t)(__float_as_uint(lo) >> 16);
+                  dp[pstride] = (uint16_t)(__float_as_uint(hi) >> 16);
+                  dp[2 * pstride] = (uint16_t)(__float_as_uint(lo + hi) >> 16);
+                }
+                dp += 3 * pstride;
+              }
+            } else {
+              // the piece that holds the last one-limb moduli and the first pairs
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const int colx = c0 + q;
+                if (colx < L1) {
+                  const float4 mc = s_mc[colx];
                   const float r = cmod_f32(__uint_as_float(y[q]), mc.x, mc.y, mc.z) + 0.0f;
-                  *dp = (uint16_t)(__float_as_uint(r) >> 16);
-                  dp += pstride;
-                }
-              } else if (c0 >= L1) {
-                // 4 two-limb pairs: moduli l = L1 + (c0 - L1) / 2 + i, planes L1 + 3 (l - L1) + {0, 1, 2}
-                const int lb = L1 + ((c0 - L1) >> 1);
-                uint16_t* dp = dst0 + (int64_t)(L1 + 3 * (lb - L1)) * pstride;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  if (c0 + 2 * i < ncols) {
-                    const float4 mc = s_mc[lb + i];
-                    // x is +0 for a zero residue; then lo, hi and lo + hi are never -0
-                    const float x = cmod2_f32(y[2 * i], y[2 * i + 1], mc.x, mc.y);
-                    float lo, hi;
-                    split128(x, lo, hi);
-                    dp[0] = (uint16_t)(__float_as_uint(lo) >> 16);
-                    dp[pstride] = (uint16_t)(__float_as_uint(hi) >> 16);
-                    dp[2 * pstride] = (uint16_t)(__float_as_uint(lo + hi) >> 16);
-                  }
-                  dp += 3 * pstride;
-                }
-              } else {
-                // the piece that holds the last one-limb moduli and the first pairs
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                  const int colx = c0 + q;
-                  if (colx < L1) {
-                    const float4 mc = s_mc[colx];
-                    const float r = cmod_f32(__uint_as_float(y[q]), mc.x, mc.y, mc.z) + 0.0f;
-                    dst0[(int64_t)colx * pstride] = (uint16_t)(__float_as_uint(r) >> 16);
-                  } else if ((q & 1) == 0 && colx < ncols) {   // a pair starts at an even column
-                    const int l = L1 + ((colx - L1) >> 1);
-                    const float4 mc = s_mc[l];
-                    const float x = cmod2_f32(y[q], y[q + 1], mc.x, mc.y);
-                    float lo, hi;
-                    split128(x, lo, hi);
-                    uint16_t* dp = dst0 + (int64_t)(L1 + 3 * (l - L1)) * pstride;
-                    dp[0] = (uint16_t)(__float_as_uint(lo) >> 16);
-                    dp[pstride] = (uint16_t)(__float_as_uint(hi) >> 16);
-                    dp[2 * pstride] = (uint16_t)(__float_as_uint(lo + hi) >> 16);
-                  }
+                  dst0[(int64_t)colx * pstride] = (uint16_t)(__float_as_uint(r) >> 16);
+                } else if ((q & 1) == 0 && colx < ncols) {   // a pair starts at an even column
+                  const int l = L1 + ((colx - L1) >> 1);
+                  const float4 mc = s_mc[l];
+                  const float x = cmod2_f32(y[q], y[q + 1], mc.x, mc.y);
+                  float lo, hi;
+                  split128(x, lo, hi);
+                  uint16_t* dp = dst0 + (int64_t)(L1 + 3 * (l - L1)) * pstride;
+                  dp[0] = (uint16_t)(__float_as_uint(lo) >> 16);
+                  dp[pstride] = (uint16_t)(__float_as_uint(hi) >> 16);
+                  dp[2 * pstride] = (uint16_t)(__float_as_uint(lo + hi) >> 16);
                 }
               }
             }
