@@ -265,13 +265,17 @@ def stage_rooflines(info, M, N, K, p, stages, workload, sustained: bool = False)
     residues: byte multiply-adds sum_b beta_b (2^(8b) mod m) over the
       ceil((t+1)/8) bytes of each integerized entry, one per modulus for the
       L1 one-limb moduli and two (the low and high table byte) for the L2
-      two-limb moduli: (M+N) K ceil((t+1)/8) (L1 + 2 L2), against the dp4a
+      two-limb moduli: (M+N) K ceil((t+1)/8) (L1 + 2 L2), two flops each
+      against the bf16 tensor peak (up to 72 bytes as warp-level f16 products,
+      beyond as a byte GEMM), or, engine 3 beyond 72 bytes, against the dp4a
       multiply-add rate.
     gemm: 2 M N K G flops of the G plane products, against the measured bf16
       tensor peak (the integer planes are exact bf16 operands); the sustained
       peak where the timed region is seconds long (`sustained`).
-    crt (CUDA-core CRT): the 32 x 32 -> 64-bit multiply-adds of
-      sum_l v_l M_l, L per output and digit of M_l: M N L ceil(bits(P)/32),
+    crt (one-kernel CRT): up to 12 digits the byte products of sum_l v_l M_l
+      and of the quotient estimate, 2 M N L 4 (ceil(bits(P)/32) + 1) flops
+      against the bf16 tensor peak; beyond the 32 x 32 -> 64-bit
+      multiply-adds, L per output and digit of M_l: M N L ceil(bits(P)/32),
       against the IMAD.WIDE rate.
     crt_sums (tensor-core CRT): the exact bf16 products of the column sums
       Y = V B that are formed, 2 M N (2L) (np - 32 s) flops with np 7-bit
@@ -310,16 +314,26 @@ def stage_rooflines(info, M, N, K, p, stages, workload, sustained: bool = False)
                      "traffic": traffic.get(name)}
 
     res_macs = (M + N) * K * math.ceil((t + 1) / 8) * (L1 + 2 * L2)
+
+    def tensor(name, kernel, flops):
+        ach = flops / (stages[name] / 1e3) / 1e12
+        out[name] = {"kernel": kernel, "bound": "tensor", "achieved": round(ach, 1), "peak": tpk, "unit": "TFLOP/s",
+                     "frac": round(ach / tpk, 4), "peak_source": tsrc, "traffic": traffic.get(name)}
+
+    # the byte products on the tensor cores: 2 flops per byte multiply-add
     if info.get("res_mode") == 2:
-        # the byte products on the tensor cores: 2 flops per byte multiply-add
-        ach = 2.0 * res_macs / (stages["residues"] / 1e3) / 1e12
-        out["residues"] = {"kernel": "k_residue_mm (integerize + residues as an exact f16 byte GEMM, kind::f16 rate)",
-                           "bound": "tensor", "achieved": round(ach, 1), "peak": tpk, "unit": "TFLOP/s",
-                           "frac": round(ach / tpk, 4), "peak_source": tsrc, "traffic": traffic.get("residues")}
+        tensor("residues", "k_residue_mm (integerize + residues as an exact f16 byte GEMM, kind::f16 rate)",
+               2.0 * res_macs)
+    elif t + 1 <= 576:
+        tensor("residues", "k_residue_frag (integerize + residues as warp-level f16 byte products + plane writes)",
+               2.0 * res_macs)
     else:
         alu("residues", "k_residue (integerize + byte-table residues + plane writes)", res_macs,
             SMS * DP4A_MACS_PER_SM_CLK * clk, "byteMAC")
-    if "crt" in stages:
+    if "crt" in stages and info["crt_digits"] <= 12:
+        tensor("crt", "k_crt_frag (CRT sum as warp-level f16 byte products + quotient correction + rounding)",
+               2.0 * M * N * L * 4 * (md + 1))
+    elif "crt" in stages:
         alu("crt", "k_crt1 / k_crt (direct CRT sum + quotient correction + rounding)", M * N * L * md,
             SMS * IMAD_WIDE_PER_SM_CLK * clk, "imad64")
     if "crt_sums" in stages:

@@ -138,7 +138,7 @@ typedef struct {
   int units;        /* (modulus, output tile) work units over all problems */
   int jobs;         /* tensor-core accumulation jobs over all problems */
   size_t workspace_bytes;
-  int crt_mode;     /* CRT path of problem 0: 0 CUDA cores, 1 tensor-core column sums in one
+  int crt_mode;     /* CRT path of problem 0: 0 a lane or lanes per output, 1 tensor-core column sums in one
                        kernel, 2 tensor-core sums of any length plus the finish (see crt_engine) */
   int res_mode;     /* residue path of problem 0: 0 in registers, 1 or 2 byte GEMM (res_engine) */
   int plane_groups; /* modulus groups the planes of problem 0 are streamed in (1: not streamed) */

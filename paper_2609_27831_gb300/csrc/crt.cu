@@ -1298,7 +1298,7 @@ __global__ void __launch_bounds__(kFinThreads) k_crt_fin_long(DevTables T, const
 // tensor-core CRT sums, R in registers: every group word and the quotient
 // estimate are loaded at once (coalesced across the block), then
 // R = (sum_g Q_g 2^(224 g) + alpha~ (2^(32 D) - P)) mod 2^(32 D), then the same
-// unrolled steps as k_crt1 (crt_finish).  Group g holds 9 words starting at
+// unrolled steps as the one-lane CRT (crt_finish).  Group g holds 9 words starting at
 // word 7 g, so word d collects word d - 7 g of group g = d / 7 and, for
 // d mod 7 < 2, word d - 7 (g - 1) of the group before.
 template <int ND>
