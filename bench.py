@@ -242,14 +242,12 @@ DP4A_MACS_PER_SM_CLK = 64 * 4
 # DRAM traffic of each stage per execute (dram__bytes_read.sum +
 # dram__bytes_write.sum over the stage's launches, averaged over the four
 # executes of one ncu capture of the committed kernels on the same workload,
-# one pass, the full size; the finish at 1024^3, p = 256 from its own
-# capture of one launch after its last change); the source summaries are
-# under profiles/.  A kernel changed since its capture is absent.
+# one pass, the full size); the source summaries are under profiles/.  A kernel changed since its capture is absent.
 NCU_TRAFFIC = {
-    "gemm_4096_p2048": {"scan": 403911680, "residues": 82033706496, "gemm": 121773933248,
-                        "crt_sums": 20133005952, "crt_finish": 11299742848},
-    "gemm_1024_p256": {"scan": 25205376, "residues": 440525568, "gemm": 562085952,
-                       "crt_finish": 125142528},
+    "gemm_4096_p2048": {"scan": 404020096, "residues": 82236858048, "gemm": 121768294080,
+                        "crt_sums": 17714513024, "crt_finish": 10712340032},
+    "gemm_1024_p256": {"scan": 25205184, "residues": 446786880, "gemm": 559872192,
+                       "crt_sums": 219710208, "crt_finish": 122059392},
 }
 
 
