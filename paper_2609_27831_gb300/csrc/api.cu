@@ -783,24 +783,37 @@ static void layout_workspace(ozaki2_plan_s* pl) {
   pl->ws_bytes = off;
 }
 
-// Automatic plane GEMM tile of a single product: CTA pairs (256 x 256) where
-// both output dimensions exceed one 128-row tile and the plane products are
-// below 1e13 flop; one SM per 128 x 256 tile for larger products, where the
-// pairs measured slower on one GB300 (1024^3 at p = 256: 0.180 vs 0.188 ms,
-// 4096^3 at p = 53: 2.07 vs 2.16 ms; 8192^3 at p = 53: 17.3 vs 17.0 ms,
-// 4096^3 at p = 2048: 82.2 vs 77.7 ms).
-static bool auto_pair_tiles(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int p) {
-  if (M <= 128 || N <= 128 || p < 2 || K <= 0 || K > kMaxK || p > kMaxP) return false;
-  // planes G from the modulus rule (Eq. 3 and Eq. crtcond), without building the plan
-  const ozaki2_opts& o = pl->opts;
-  const int t = o.t_bits > 0 ? o.t_bits : p + o.guard_bits + ceil_log2(K);
-  Big P;
-  const int L = modulus_prefix(K, t, 0, &P);
-  if (L < 0) return false;
-  const int L1 = std::min(L, one_limb_count());
-  const double G = L1 + 3.0 * (L - L1);
-  return 2.0 * (double)M * (double)N * (double)K * G < 1e13;
-}
+// Automatic plane GEMM tile: CTA pairs (256 x 256) where they cover the outputs with
+// at most 12 % more tile area (weighted by K) than 128 x 256 tiles, where the plane
+// products fill the 152 SMs at least four times over, and below 1e13 flop.  Measured
+// on one GB300, one SM and pairs, plane GEMM stage in ms: 1024^3 p = 256 0.156 and
+// 0.137, 1531 x 1093 x 1777 p = 512 1.50 and 1.15, 64 uneven products (1.08 times
+// the area) 8.49 and 7.89; equal at 2.8 to 5.4 rounds (256^3 p = 512, 512^3 p = 256);
+// below, 384^3 p = 53 0.0143 and 0.0185, and with 20 % more area 611 x 347 x 923
+// p = 113 0.039 and 0.045.  Beyond 1e13 flop the power cap evens them out: 8192^3
+// p = 53 20.1 and 20.0 ms for the product, 4096^3 p = 2048 113.2 and 115.0.
+struct TileLoad {
+  double rounds = 0, one = 0, two = 0, flops = 0;
+  // a product's planes G from the modulus rule (Eq. 3 and Eq. crtcond), without building it
+  void add(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts& o, const PlanExtra& ex = PlanExtra()) {
+    if (M <= 0 || N <= 0 || K <= 0 || M > INT_MAX || N > INT_MAX || K > kMaxK || p < 2 || p > kMaxP) return;
+    const int64_t inner = std::max<int64_t>(K, ex.inner);
+    const int t = ex.force_t > 0 ? ex.force_t : (o.t_bits > 0 ? o.t_bits : p + o.guard_bits + ceil_log2(inner));
+    Big P;
+    const int L = modulus_prefix(inner, t, ex.force_L, &P);
+    if (L < 0) return;
+    const int L1 = std::min(L, one_limb_count());
+    const double G = L1 + 3.0 * (L - L1);
+    const double n1 = G * (double)((M + 127) / 128) * (double)((N + 255) / 256);
+    const double n2 = G * (double)((M + 255) / 256) * (double)((N + 255) / 256);
+    rounds += n1 / 152;
+    flops += 2.0 * G * (double)M * (double)N * (double)K;
+    one += n1 * (double)K;
+    two += 2 * n2 * (double)K;
+  }
+  bool pairs() const { return rounds >= 4 && two <= 1.12 * one && flops < 1e13; }
+};
+static bool auto_tile(const ozaki2_plan_s* pl) { return pl->opts.gemm_tile == 0 && pl->opts.engine == OZ2_ENGINE_TC; }
 
 static int new_plan(const ozaki2_opts* opts, ozaki2_plan_s** res) {
   auto* pl = new (std::nothrow) ozaki2_plan_s();
@@ -1688,6 +1701,11 @@ int plan_create_ex(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts* op
   if (rc) return rc;
   pl->no_stream = true;                          // the binary64 mode keeps every plane for the backward
   try {
+    if (auto_tile(pl)) {
+      TileLoad tl;
+      tl.add(M, N, K, p, pl->opts, ex);
+      pl->tile2 = tl.pairs();
+    }
     rc = build_problem(pl, M, N, K, p, &ex);
   } catch (const std::bad_alloc&) {
     rc = OZ2_ENOMEM;
@@ -1758,8 +1776,12 @@ int ozaki2_plan_create(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts
   ozaki2_plan_s* pl = nullptr;
   int rc = new_plan(opts, &pl);
   if (rc) return rc;
-  if (pl->opts.gemm_tile == 0 && pl->opts.engine == OZ2_ENGINE_TC) pl->tile2 = auto_pair_tiles(pl, M, N, K, p);
   try {
+    if (auto_tile(pl)) {
+      TileLoad tl;
+      tl.add(M, N, K, p, pl->opts);
+      pl->tile2 = tl.pairs();
+    }
     rc = build_problem(pl, M, N, K, p);
     if (!rc) rc = plan_groups(pl);
   } catch (const std::bad_alloc&) {
@@ -1801,6 +1823,12 @@ int ozaki2_plan_create_batched_ex(int count, const ozaki2_problem* shapes, const
     }
   }
   try {
+    if (auto_tile(pl)) {
+      TileLoad tl;
+      for (int i = 0; i < count; ++i)
+        tl.add(shapes[i].M, shapes[i].N, shapes[i].K, shapes[i].p, po.empty() ? pl->opts : po[i]);
+      pl->tile2 = tl.pairs();
+    }
     for (int i = 0; i < count && !rc; ++i)
       rc = build_problem(pl, shapes[i].M, shapes[i].N, shapes[i].K, shapes[i].p, nullptr, po.empty() ? nullptr : &po[i]);
   } catch (const std::bad_alloc&) {
@@ -1818,11 +1846,15 @@ int ozaki2_plan_create_complex(int64_t M, int64_t N, int64_t K, int p, const oza
   ozaki2_plan_s* pl = nullptr;
   int rc = new_plan(opts, &pl);
   if (rc) return rc;
-  if (pl->opts.gemm_tile == 0 && pl->opts.engine == OZ2_ENGINE_TC) pl->tile2 = auto_pair_tiles(pl, M, N, K, p);
   pl->complex3m = true;
   PlanExtra ex;
   ex.inner = 2 * K;                              // |Cr_hat|, |Ci_hat| <= 2K 2^(2t)
   try {
+    if (auto_tile(pl)) {
+      TileLoad tl;
+      for (int i = 0; i < 3; ++i) tl.add(M, N, K, p, pl->opts, ex);
+      pl->tile2 = tl.pairs();
+    }
     for (int i = 0; i < 3 && !rc; ++i) rc = build_problem(pl, M, N, K, p, &ex);
   } catch (const std::bad_alloc&) {
     rc = OZ2_ENOMEM;
