@@ -248,7 +248,8 @@ int cache_retire(ozaki2_cache_s* c) {
   return OZ2_OK;
 }
 
-int cache_build(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2_cache_s** out) {
+// A cache with its forward plan: host work only.
+int cache_plan(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2_cache_s** out) {
   if (M <= 0 || N <= 0 || K <= 0) return OZ2_EINVAL;
   if (M > INT32_MAX / 2 || N > INT32_MAX / 2 || K > INT32_MAX / 2) return OZ2_ERANGE;
   auto* c = new (std::nothrow) ozaki2_cache_s();
@@ -262,6 +263,14 @@ int cache_build(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2
   int rc = plan_create_ex(M, N, K, 53, &c->opts, ex, &c->fwd);
   if (!rc) rc = plan_query(c->fwd, &c->ff);
   if (rc) { cache_release(c); return rc; }
+  *out = c;
+  return OZ2_OK;
+}
+
+int cache_build(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2_cache_s** out) {
+  ozaki2_cache_s* c = nullptr;
+  const int rc = cache_plan(M, N, K, opts, &c);
+  if (rc) return rc;
   const size_t bytes = al(c->ff.ws_bytes) + MpBuf::bytes((int)M, (int)K) + MpBuf::bytes((int)K, (int)N);
   if (dev_malloc(&c->mem, bytes) != cudaSuccess) { c->mem = nullptr; cache_release(c); return OZ2_ENOMEM; }
   c->fwd_bytes = bytes;
@@ -377,15 +386,16 @@ int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t l
     ozaki2_opts o;
     if (opts) o = *opts;
     else ozaki2_opts_default(&o);
+    if (cache_out) *cache_out = nullptr;
+    if (!A || !B || !Cd || lda < K || ldb < N || ldc < N) {
+      // refused on the host; a size or option that no plan takes is named first
+      ozaki2_cache_s* c = nullptr;
+      const int rc = cache_plan(M, N, K, &o, &c);
+      if (rc) return rc;
+      cache_release(c);
+      return OZ2_EINVAL;
+    }
     if (cache_out) {
-      *cache_out = nullptr;
-      if (!A || !B || !Cd || lda < K || ldb < N || ldc < N) {      // refused before a retired cache is taken
-        ozaki2_cache_s* c = nullptr;
-        const int rc = cache_build(M, N, K, &o, &c);
-        if (rc) return rc;
-        cache_release(c);
-        return OZ2_EINVAL;
-      }
       auto key = cache_key(M, N, K, o);
       ozaki2_cache_s* c = pool_take(key, s);
       if (!c) {

@@ -241,6 +241,28 @@ def test_plane_group_option_errors(ozk):
         assert ozk.Plan((200, 150, 300, 256), **kw).info["plane_groups"] == 1
 
 
+@pytest.mark.parametrize("keep", [True, False])
+def test_refused_binary64_forwards_allocate_nothing(ozk, keep):
+    """A null operand or a short stride is refused on the host: OZ2_EINVAL for
+    a shape whose workspace no device holds (and here, without a device); a
+    size or an option that no plan takes keeps its own code."""
+    lib, n = ozk.lib(), 100000
+
+    def fwd(M=n, K=n, a=256, b=256, c=256, ld=(n, n, n), **kw):
+        h = C.c_void_p()
+        st = lib.ozaki2_dgemm_fwd(M, n, K, a, ld[0], b, ld[1], c, ld[2], C.byref(ozk.opts(**kw)),
+                                  C.byref(h) if keep else None, None)
+        assert not h.value
+        return st
+
+    for kw in ({"a": None}, {"b": None}, {"c": None}, {"ld": (n - 1, n, n)}, {"ld": (n, n - 1, n)},
+               {"ld": (n, n, n - 1)}):
+        assert fwd(**kw) == ozk._lib.OZ2_EINVAL, kw
+    assert fwd(a=None, K=133001) == ozk._lib.OZ2_ERANGE
+    assert fwd(a=None, M=0) == ozk._lib.OZ2_EINVAL
+    assert fwd(a=None, engine=7) == ozk._lib.OZ2_EINVAL
+
+
 def test_injected_host_allocation_failure(ozk):
     """A host allocation failure while a plan is built is reported as
     OZ2_ENOMEM (nothing aborts, nothing half-made is kept); the next call
