@@ -359,7 +359,7 @@ OZ2_API int ozaki2_gemm_batched(int count, const ozaki2_problem* probs, const oz
                         void* stream);
 
 /* Free the plans and workspaces cached by ozaki2_gemm / ozaki2_gemm_batched /
-   ozaki2_zgemm, and the binary64 caches kept by ozaki2_cache_destroy. */
+   ozaki2_zgemm, and the binary64 plans kept by ozaki2_cache_destroy. */
 OZ2_API int ozaki2_release_cache(void);
 
 /* Synchronise `stream` and read the plan's device status word:
@@ -389,6 +389,10 @@ OZ2_API int ozaki2_last_crt_split(ozaki2_plan plan, float ms[2]);
  * three products.  Results are rounded to nearest-even binary64.
  * ------------------------------------------------------------------------- */
 
+/* Device memory from the caller's own allocator: `bytes` of it, 256-byte aligned,
+   or NULL (OZ2_ENOMEM). */
+typedef void* (*ozaki2_alloc_fn)(size_t bytes, void* user);
+
 /* Forward.  cache_out may be NULL (no backward); else *cache_out receives a
    library-owned cache (device memory) to pass to ozaki2_dgemm_bwd. */
 OZ2_API int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda,
@@ -400,12 +404,29 @@ OZ2_API int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, i
 OZ2_API int ozaki2_dgemm_bwd(ozaki2_cache cache, const double* dC, int64_t lddc, double* dA,
                      int64_t ldda, double* dB, int64_t lddb, void* stream);
 
-/* Give a cache back.  The library may keep its memory for the next
-   ozaki2_dgemm_fwd of the same shape and options on the same device (at most 32
-   caches and an eighth of the device's memory, none while less than a quarter of
-   it is free; freed by ozaki2_release_cache and before an allocation of the
-   library fails); the stream of that call waits for this cache's last run. */
+/* The same, working in memory of the caller's: `alloc` (NULL: as above) is called
+   once for all that the call needs.  The forward's memory holds the planes and
+   stays the cache's until ozaki2_cache_destroy (library memory is used where
+   cache_out is NULL); the backward's is needed until its work on `stream` is done.
+   The caller keeps each from reuse until the last run with it has finished. */
+OZ2_API int ozaki2_dgemm_fwd_alloc(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda,
+                                   const double* B, int64_t ldb, double* C, int64_t ldc,
+                                   const ozaki2_opts* opts, ozaki2_alloc_fn alloc, void* user,
+                                   ozaki2_cache* cache_out, void* stream);
+OZ2_API int ozaki2_dgemm_bwd_alloc(ozaki2_cache cache, const double* dC, int64_t lddc, double* dA,
+                                   int64_t ldda, double* dB, int64_t lddb, ozaki2_alloc_fn alloc, void* user,
+                                   void* stream);
+
+/* Give a cache back, and the library's memory that it worked in.  The library may
+   keep its plans and their device tables for the next ozaki2_dgemm_fwd of the same
+   shape and options on the same device (per device at most 32 caches and 256 MiB
+   of tables, the oldest freed first; all freed by ozaki2_release_cache and before
+   an allocation of the library fails); the stream of that call waits for this
+   cache's last run. */
 OZ2_API int ozaki2_cache_destroy(ozaki2_cache cache);
+
+/* Caches kept so, over all devices, and the device memory of their tables. */
+OZ2_API int ozaki2_retired_caches(int* count, size_t* bytes);
 
 /* ---------------------------------------------------------------------------
  * Measurement aid (no counterpart in the paper): the throughput of the

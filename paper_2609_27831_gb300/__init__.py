@@ -17,7 +17,7 @@ from . import _lib as L
 from ._lib import OzakiError, check, lib, opts  # noqa: F401
 
 __all__ = ["MPMatrix", "Plan", "ComplexPlan", "Graph", "gemm", "gemm_batched", "zgemm", "OzakiError", "lib",
-           "opts"]
+           "opts", "release_cache"]
 
 
 def _stream_handle(stream) -> int:
@@ -277,3 +277,9 @@ def gemm_batched(pairs, ps=None, stream=None, **kw):
     check(lib().ozaki2_gemm_batched(len(pairs), arr, C.byref(o), _stream_handle(stream)),
           "ozaki2_gemm_batched")
     return outs
+
+
+def release_cache() -> None:
+    """Free the plans and workspaces that the library keeps between calls: those of ``gemm``,
+    ``gemm_batched`` and ``zgemm``, and the plans of past binary64 products."""
+    check(lib().ozaki2_release_cache(), "ozaki2_release_cache")

@@ -42,6 +42,9 @@ class Problem(C.Structure):
                 ("A", Mat), ("B", Mat), ("C", Mat)]
 
 
+ALLOC_FN = C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p)
+
+
 class OzakiError(RuntimeError):
     def __init__(self, status: int, what: str):
         self.status = status
@@ -104,7 +107,13 @@ _SIGS = {
                                     C.POINTER(C.c_void_p), C.c_void_p]),
     "ozaki2_dgemm_bwd": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64,
                                     C.c_void_p, C.c_int64, C.c_void_p]),
+    "ozaki2_dgemm_fwd_alloc": (C.c_int, [C.c_int64, C.c_int64, C.c_int64, C.c_void_p, C.c_int64,
+                                          C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.POINTER(Opts),
+                                          ALLOC_FN, C.c_void_p, C.POINTER(C.c_void_p), C.c_void_p]),
+    "ozaki2_dgemm_bwd_alloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64,
+                                          C.c_void_p, C.c_int64, ALLOC_FN, C.c_void_p, C.c_void_p]),
     "ozaki2_cache_destroy": (C.c_int, [C.c_void_p]),
+    "ozaki2_retired_caches": (C.c_int, [C.POINTER(C.c_int), C.POINTER(C.c_size_t)]),
     "ozaki2_probe_mma_s8": (C.c_int, [C.c_int, C.c_int, C.c_void_p, C.POINTER(C.c_double), C.c_void_p]),
 }
 

@@ -5,7 +5,8 @@ The forward calls ``ozaki2_dgemm_fwd`` and keeps the returned cache of int8
 residue planes; the hand-written backward calls ``ozaki2_dgemm_bwd``, which
 computes dA = dC B^T and dB = A^T dC through the same exact path while reusing
 the forward's residue planes of B and A instead of recomputing them.  All
-arithmetic runs in the library's CUDA kernels.
+arithmetic runs in the library's CUDA kernels, in memory of torch's allocator:
+the planes' until the graph node dies, the backward's for its call.
 """
 from __future__ import annotations
 
@@ -16,11 +17,23 @@ import torch
 from . import _lib as L
 
 
-class _Cache:
-    """Owns one library cache handle (freed when the graph node dies)."""
+def _allocator(device: torch.device, out: list) -> L.ALLOC_FN:
+    """A function that gives one library call memory of torch's allocator and leaves the
+    tensor in ``out`` (no reference cycle: the memory goes back with its last user)."""
+    def alloc(nbytes, _user):
+        try:
+            out.append(torch.empty(nbytes, dtype=torch.uint8, device=device))
+        except torch.OutOfMemoryError:
+            return None                      # the call returns OZ2_ENOMEM
+        return out[-1].data_ptr()
+    return L.ALLOC_FN(alloc)
 
-    def __init__(self, handle: C.c_void_p):
-        self.h = handle
+
+class _Cache:
+    """Owns one library cache handle (freed when the graph node dies) and the memory of its planes."""
+
+    def __init__(self, handle: C.c_void_p, buf: torch.Tensor):
+        self.h, self.buf = handle, buf
 
     def __del__(self):
         if getattr(self, "h", None) and self.h.value:
@@ -46,12 +59,13 @@ class OzakiMatmul(torch.autograd.Function):
         Cm = torch.empty((M, N), dtype=torch.float64, device=A.device)
         h = C.c_void_p()
         need = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
-        st = L.lib().ozaki2_dgemm_fwd(M, N, K, A.data_ptr(), K, B.data_ptr(), N, Cm.data_ptr(), N,
-                                      C.byref(opts) if opts is not None else None,
-                                      C.byref(h) if need else None,
-                                      torch.cuda.current_stream(A.device).cuda_stream)
+        mem = []
+        st = L.lib().ozaki2_dgemm_fwd_alloc(M, N, K, A.data_ptr(), K, B.data_ptr(), N, Cm.data_ptr(), N,
+                                            C.byref(opts) if opts is not None else None, _allocator(A.device, mem),
+                                            None, C.byref(h) if need else None,
+                                            torch.cuda.current_stream(A.device).cuda_stream)
         L.check(st, "ozaki2_dgemm_fwd")
-        ctx.cache = _Cache(h) if need else None
+        ctx.cache = _Cache(h, mem[0]) if need else None
         ctx.shape = (M, N, K)
         return Cm
 
@@ -61,10 +75,13 @@ class OzakiMatmul(torch.autograd.Function):
         dC = dC.to(torch.float64).contiguous()
         dA = torch.empty((M, K), dtype=torch.float64, device=dC.device) if ctx.needs_input_grad[0] else None
         dB = torch.empty((K, N), dtype=torch.float64, device=dC.device) if ctx.needs_input_grad[1] else None
-        st = L.lib().ozaki2_dgemm_bwd(ctx.cache.h, dC.data_ptr(), N,
-                                      dA.data_ptr() if dA is not None else None, K,
-                                      dB.data_ptr() if dB is not None else None, N,
-                                      torch.cuda.current_stream(dC.device).cuda_stream)
+        stream = torch.cuda.current_stream(dC.device)
+        mem = []                                 # back to torch when this call returns
+        ctx.cache.buf.record_stream(stream)      # read here, whatever stream the forward ran on
+        st = L.lib().ozaki2_dgemm_bwd_alloc(ctx.cache.h, dC.data_ptr(), N,
+                                            dA.data_ptr() if dA is not None else None, K,
+                                            dB.data_ptr() if dB is not None else None, N,
+                                            _allocator(dC.device, mem), None, stream.cuda_stream)
         L.check(st, "ozaki2_dgemm_bwd")
         return dA, dB, None
 

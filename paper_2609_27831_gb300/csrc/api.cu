@@ -236,6 +236,7 @@ struct LaunchBlock {
 struct DevState {
   int device = -1, sms = 0;
   void* mem = nullptr;
+  size_t mem_bytes = 0;
   DevTables tab{};
   const Unit* unsorted = nullptr;
   ListRef scan_rows, scan_cols, simt, s8;
@@ -1332,6 +1333,7 @@ static int upload(ozaki2_plan_s* pl) {
     return OZ2_ECUDA;
   }
   d.mem = mem;
+  d.mem_bytes = ti.b.img.size();
   d.device = dev;
   install_table_image(pl, ti, static_cast<uint8_t*>(mem));
   if (pl->opts.timing) {
@@ -1723,6 +1725,13 @@ int plan_query(ozaki2_plan pl, PlanFacts* f) {
   f->off_e = h.off_e; f->off_f = h.off_f; f->off_pa = h.off_pa; f->off_pb = h.off_pb;
   f->ws_bytes = pl->ws_bytes;
   return OZ2_OK;
+}
+
+size_t plan_device_bytes(ozaki2_plan pl) {
+  if (!pl) return 0;
+  size_t n = pl->dev.mem_bytes;
+  for (const LaunchBlock& lb : pl->lbs) n += lb.d_mem ? lb.bytes : 0;
+  return n;
 }
 
 int plan_run(ozaki2_plan pl, const ozaki2_problem* q, void* ws, size_t ws_bytes, cudaStream_t s) {

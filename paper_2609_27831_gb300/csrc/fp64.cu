@@ -151,8 +151,8 @@ struct ozaki2_cache_s {
   ozaki2_plan fwd = nullptr, bwd_a = nullptr, bwd_b = nullptr;
   oz2::PlanFacts ff{}, fa{}, fb{};
   void* mem = nullptr;          // fwd workspace + A/B conversions
-  void* mem_bwd = nullptr;      // backward workspaces + dC conversion
-  size_t fwd_bytes = 0, bwd_bytes = 0;
+  bool own_mem = false;         // mem is the library's (else its caller's)
+  void* mem_bwd = nullptr;      // backward workspaces + dC conversion, the library's
   oz2::MpBuf a, b;
   std::vector<int64_t> key;     // device, shape and options: what a later forward must match to take it over
   cudaEvent_t done = nullptr;   // recorded after every run with this cache
@@ -161,33 +161,44 @@ struct ozaki2_cache_s {
 namespace oz2 {
 namespace {
 
+// Free the memory that a forward and a backward work in, or let go of its caller's.
+void cache_drop_memory(ozaki2_cache_s* c) {
+  if (c->own_mem || c->mem_bwd) cudaDeviceSynchronize();
+  if (c->own_mem) cudaFree(c->mem);
+  if (c->mem_bwd) cudaFree(c->mem_bwd);
+  c->mem = c->mem_bwd = nullptr;
+  c->own_mem = false;
+}
+
 int cache_release(ozaki2_cache_s* c) {
   if (!c) return OZ2_EINVAL;
-  if (c->mem || c->mem_bwd) cudaDeviceSynchronize();
+  if (c->mem || c->done) cudaDeviceSynchronize();    // the plans' tables are read by their runs
+  cache_drop_memory(c);
   if (c->done) cudaEventDestroy(c->done);
   if (c->fwd) ozaki2_plan_destroy(c->fwd);
   if (c->bwd_a) ozaki2_plan_destroy(c->bwd_a);
   if (c->bwd_b) ozaki2_plan_destroy(c->bwd_b);
-  if (c->mem) cudaFree(c->mem);
-  if (c->mem_bwd) cudaFree(c->mem_bwd);
   delete c;
   return OZ2_OK;
 }
 
-// Retired caches (plans, workspaces and conversion buffers), kept for the next
-// forward of the same shape and options on the same device: making one takes
-// several device and pinned allocations, table uploads and a device-wide wait
-// when it is freed (a 4096^3 forward and backward: 8 of 20.1 ms).  Bounded: at
-// most kPoolCaches caches and an eighth of the device's memory, the oldest freed
-// first, and none kept while less than a quarter of the device's memory is
-// free; all freed by ozaki2_release_cache and when a library allocation fails.
-// A cache that is taken over makes the new stream wait for `done`, so its
-// buffers are not rewritten before their last readers, whatever their stream.
+// Retired caches, kept for the next forward of the same shape and options on the
+// same device: their plans with the device tables and pinned launch blocks, whose
+// making takes several allocations, table uploads and a device-wide wait; never the
+// memory that the products work in, which goes back when a cache is retired.
+// Bounded per device: at most kPoolCaches caches and kPoolBytes of tables, the
+// oldest freed first; all freed by ozaki2_release_cache and when a library
+// allocation fails.  A cache that is taken over makes the new stream wait for
+// `done`, so its tables and launch blocks are not rewritten before their last
+// readers, whatever their stream.
 constexpr size_t kPoolCaches = 32;
+constexpr size_t kPoolBytes = (size_t)256 << 20;
 std::mutex g_pool_mu;
 std::list<ozaki2_cache_s*> g_pool;   // oldest first
 
-size_t cache_bytes(const ozaki2_cache_s* c) { return c->fwd_bytes + c->bwd_bytes; }
+size_t cache_table_bytes(const ozaki2_cache_s* c) {
+  return plan_device_bytes(c->fwd) + plan_device_bytes(c->bwd_a) + plan_device_bytes(c->bwd_b);
+}
 
 std::vector<int64_t> cache_key(int64_t M, int64_t N, int64_t K, const ozaki2_opts& o) {
   int dev = -1;
@@ -225,27 +236,40 @@ ozaki2_cache_s* pool_take(const std::vector<int64_t>& key, cudaStream_t s) {
   return c;
 }
 
-// Keep a cache that its owner has given back, or free it.
+// Keep the plans of a cache that its owner has given back, or free it.
 int cache_retire(ozaki2_cache_s* c) {
   if (!c) return OZ2_EINVAL;
-  size_t free_b = 0, total_b = 0;
   int dev = -1;
   if (!c->done || c->key.empty() || cudaGetDevice(&dev) != cudaSuccess || c->key[0] != dev ||
-      cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || free_b < total_b / 4 || cache_bytes(c) > total_b / 8)
+      cache_table_bytes(c) > kPoolBytes)
     return cache_release(c);
+  cache_drop_memory(c);
   std::list<ozaki2_cache_s*> out;
   {
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    size_t held = cache_bytes(c);
-    for (const ozaki2_cache_s* q : g_pool) held += cache_bytes(q);
-    while (!g_pool.empty() && (held > total_b / 8 || g_pool.size() + 1 > kPoolCaches)) {
-      held -= cache_bytes(g_pool.front());
-      out.splice(out.end(), g_pool, g_pool.begin());
-    }
     g_pool.push_back(c);
+    size_t n = 0, held = 0;                          // of this device, newest first
+    for (auto it = g_pool.end(); it != g_pool.begin();) {
+      --it;
+      if ((*it)->key[0] != dev) continue;
+      ++n;
+      held += cache_table_bytes(*it);
+      if (n > kPoolCaches || held > kPoolBytes) {
+        out.push_back(*it);
+        it = g_pool.erase(it);
+      }
+    }
   }
   for (ozaki2_cache_s* q : out) cache_release(q);
   return OZ2_OK;
+}
+
+// Memory from the caller where it gives a function for it, else the library's.
+int work_malloc(size_t bytes, ozaki2_alloc_fn alloc, void* user, void** p) {
+  if (alloc) *p = alloc(bytes, user);
+  else if (dev_malloc(p, bytes) != cudaSuccess) *p = nullptr;
+  if (!*p) return OZ2_ENOMEM;
+  return (reinterpret_cast<uintptr_t>(*p) & 255u) ? OZ2_EINVAL : OZ2_OK;
 }
 
 // A cache with its forward plan: host work only.
@@ -267,17 +291,15 @@ int cache_plan(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2_
   return OZ2_OK;
 }
 
-int cache_build(int64_t M, int64_t N, int64_t K, const ozaki2_opts* opts, ozaki2_cache_s** out) {
-  ozaki2_cache_s* c = nullptr;
-  const int rc = cache_plan(M, N, K, opts, &c);
+int ensure_fwd_memory(ozaki2_cache_s* c, ozaki2_alloc_fn alloc, void* user) {
+  const int M = (int)c->M, N = (int)c->N, K = (int)c->K;
+  const size_t ws = al(c->ff.ws_bytes);
+  const int rc = work_malloc(ws + MpBuf::bytes(M, K) + MpBuf::bytes(K, N), alloc, user, &c->mem);
   if (rc) return rc;
-  const size_t bytes = al(c->ff.ws_bytes) + MpBuf::bytes((int)M, (int)K) + MpBuf::bytes((int)K, (int)N);
-  if (dev_malloc(&c->mem, bytes) != cudaSuccess) { c->mem = nullptr; cache_release(c); return OZ2_ENOMEM; }
-  c->fwd_bytes = bytes;
+  c->own_mem = !alloc;
   auto* base = static_cast<uint8_t*>(c->mem);
-  c->a.place(base + al(c->ff.ws_bytes), (int)M, (int)K);
-  c->b.place(base + al(c->ff.ws_bytes) + MpBuf::bytes((int)M, (int)K), (int)K, (int)N);
-  *out = c;
+  c->a.place(base + ws, M, K);
+  c->b.place(base + ws + MpBuf::bytes(M, K), K, N);
   return OZ2_OK;
 }
 
@@ -296,30 +318,33 @@ int run_fwd(ozaki2_cache_s* c, const double* A, int64_t lda, const double* B, in
 }
 
 int ensure_bwd(ozaki2_cache_s* c) {
-  if (c->mem_bwd) return OZ2_OK;
+  if (c->bwd_b) return OZ2_OK;
   PlanExtra ea;
   ea.force_t = c->ff.t; ea.force_L = c->ff.L; ea.kind = 1; ea.skip_b = true;
-  int rc = plan_create_ex(c->M, c->K, c->N, 53, &c->opts, ea, &c->bwd_a);   // dA = D1 (M x N) * B_hat^T
+  int rc = c->bwd_a ? OZ2_OK : plan_create_ex(c->M, c->K, c->N, 53, &c->opts, ea, &c->bwd_a);   // dA = D1 (M x N) * B_hat^T
   if (!rc) rc = plan_query(c->bwd_a, &c->fa);
   PlanExtra eb;
   eb.force_t = c->ff.t; eb.force_L = c->ff.L; eb.kind = 1; eb.skip_a = true;
   if (!rc) rc = plan_create_ex(c->K, c->N, c->M, 53, &c->opts, eb, &c->bwd_b);   // dB = A_hat^T * D2 (M x N)
   if (!rc) rc = plan_query(c->bwd_b, &c->fb);
-  if (rc) return rc;
-  const size_t bytes = al(c->fa.ws_bytes) + al(c->fb.ws_bytes) + MpBuf::bytes((int)c->M, (int)c->N);
-  if (dev_malloc(&c->mem_bwd, bytes) != cudaSuccess) { c->mem_bwd = nullptr; return OZ2_ENOMEM; }
-  c->bwd_bytes = bytes;
-  return OZ2_OK;
+  return rc;
 }
 
 int run_bwd(ozaki2_cache_s* c, const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB,
-            int64_t lddb, cudaStream_t s) {
+            int64_t lddb, ozaki2_alloc_fn alloc, void* user, cudaStream_t s) {
   if (!dC || lddc < c->N) return OZ2_EINVAL;
   if ((dA && ldda < c->K) || (dB && lddb < c->N)) return OZ2_EINVAL;
   int rc = ensure_bwd(c);
   if (rc) return rc;
   auto* fw = static_cast<uint8_t*>(c->mem);
-  auto* bw = static_cast<uint8_t*>(c->mem_bwd);
+  void* mem = alloc ? nullptr : c->mem_bwd;
+  if (!mem) {
+    const size_t bytes = al(c->fa.ws_bytes) + al(c->fb.ws_bytes) + MpBuf::bytes((int)c->M, (int)c->N);
+    rc = work_malloc(bytes, alloc, user, &mem);
+    if (rc) return rc;
+    if (!alloc) c->mem_bwd = mem;
+  }
+  auto* bw = static_cast<uint8_t*>(mem);
   uint8_t* ws_a = bw;
   uint8_t* ws_b = bw + al(c->fa.ws_bytes);
   MpBuf d;
@@ -378,9 +403,9 @@ using namespace oz2;
 
 extern "C" {
 
-int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B,
-                     int64_t ldb, double* Cd, int64_t ldc, const ozaki2_opts* opts, ozaki2_cache* cache_out,
-                     void* stream) {
+int ozaki2_dgemm_fwd_alloc(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B,
+                           int64_t ldb, double* Cd, int64_t ldc, const ozaki2_opts* opts, ozaki2_alloc_fn alloc,
+                           void* user, ozaki2_cache* cache_out, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   try {
     ozaki2_opts o;
@@ -399,10 +424,11 @@ int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t l
       auto key = cache_key(M, N, K, o);
       ozaki2_cache_s* c = pool_take(key, s);
       if (!c) {
-        const int rc = cache_build(M, N, K, &o, &c);
+        const int rc = cache_plan(M, N, K, &o, &c);
         if (rc) return rc;
       }
-      const int rc = run_fwd(c, A, lda, B, ldb, Cd, ldc, s);
+      int rc = ensure_fwd_memory(c, alloc, user);
+      if (!rc) rc = run_fwd(c, A, lda, B, ldb, Cd, ldc, s);
       if (rc) { cache_release(c); return rc; }
       c->key.clear();                                // kept later only if its runs are recorded
       if (!capturing(s)) {
@@ -420,8 +446,10 @@ int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t l
     auto it = g_nocache.find(key);
     if (it == g_nocache.end()) {
       ozaki2_cache_s* c = nullptr;
-      const int rc = cache_build(M, N, K, &o, &c);
+      int rc = cache_plan(M, N, K, &o, &c);
       if (rc) return rc;
+      rc = ensure_fwd_memory(c, nullptr, nullptr);
+      if (rc) { cache_release(c); return rc; }
       it = g_nocache.emplace(key, c).first;
     }
     return run_fwd(it->second, A, lda, B, ldb, Cd, ldc, s);
@@ -430,14 +458,20 @@ int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t l
   }
 }
 
-int ozaki2_dgemm_bwd(ozaki2_cache cache, const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB,
-                     int64_t lddb, void* stream) {
+int ozaki2_dgemm_fwd(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B,
+                     int64_t ldb, double* Cd, int64_t ldc, const ozaki2_opts* opts, ozaki2_cache* cache_out,
+                     void* stream) {
+  return ozaki2_dgemm_fwd_alloc(M, N, K, A, lda, B, ldb, Cd, ldc, opts, nullptr, nullptr, cache_out, stream);
+}
+
+int ozaki2_dgemm_bwd_alloc(ozaki2_cache cache, const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB,
+                           int64_t lddb, ozaki2_alloc_fn alloc, void* user, void* stream) {
   if (!cache) return OZ2_EINVAL;
   try {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // ordered after the cache's earlier runs, and recorded for the later ones
     const bool ordered = !cache->key.empty() && !capturing(s) && cudaStreamWaitEvent(s, cache->done, 0) == cudaSuccess;
-    const int rc = run_bwd(cache, dC, lddc, dA, ldda, dB, lddb, s);
+    const int rc = run_bwd(cache, dC, lddc, dA, ldda, dB, lddb, alloc, user, s);
     if (!ordered || cudaEventRecord(cache->done, s) != cudaSuccess) cache->key.clear();
     return rc;
   } catch (const std::bad_alloc&) {
@@ -445,6 +479,20 @@ int ozaki2_dgemm_bwd(ozaki2_cache cache, const double* dC, int64_t lddc, double*
   }
 }
 
+int ozaki2_dgemm_bwd(ozaki2_cache cache, const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB,
+                     int64_t lddb, void* stream) {
+  return ozaki2_dgemm_bwd_alloc(cache, dC, lddc, dA, ldda, dB, lddb, nullptr, nullptr, stream);
+}
+
 int ozaki2_cache_destroy(ozaki2_cache cache) { return cache_retire(cache); }
+
+int ozaki2_retired_caches(int* count, size_t* bytes) {
+  if (!count || !bytes) return OZ2_EINVAL;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  *count = (int)g_pool.size();
+  *bytes = 0;
+  for (const ozaki2_cache_s* c : g_pool) *bytes += cache_table_bytes(c);
+  return OZ2_OK;
+}
 
 }  // extern "C"

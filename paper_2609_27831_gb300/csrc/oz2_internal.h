@@ -210,7 +210,7 @@ cudaError_t launch_residues_mm(const DevTables& t, const int32_t* tiles, int nti
 void residue_mm_geometry(int kpad, int npad, int* cw, int* nabuf);
 int residue_mm_smem_bytes(int cw_max, int lmax, int tcols, int* stages);
 
-// cudaMalloc that frees the binary64 mode's retired caches and tries once more
+// cudaMalloc that frees the binary64 mode's retired caches (their tables) and tries once more
 // before it reports a failure.
 cudaError_t dev_malloc(void** p, size_t bytes);
 void release_retired_caches();
@@ -231,6 +231,7 @@ struct PlanFacts {
 int plan_create_ex(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts* opts,
                    const PlanExtra& ex, ozaki2_plan* out);
 int plan_query(ozaki2_plan pl, PlanFacts* f);
+size_t plan_device_bytes(ozaki2_plan pl);   // device tables and launch blocks held (0: null plan)
 int plan_run(ozaki2_plan pl, const ozaki2_problem* q, void* ws, size_t ws_bytes, cudaStream_t s);
 
 // Residue kernel W16 classes and CRT lane-group classes (host picks per problem).
