@@ -274,21 +274,29 @@ __device__ __forceinline__ void epi_chunk(const Job& j, const EpiConst& e, uint3
 
 // The epilogue of one job over NC chunks of 32 columns at tbase, the TMEM
 // load of each chunk in flight while the one before it is reduced.  Ends
-// with every TMEM store of the job complete.
+// with every TMEM store of the job complete.  Outputs of up to kNarrow columns
+// take the chunks that hold any of them: the others cost as much as those, most of
+// the stage for a few vectors (plane GEMMs with every chunk and so, ms: 4578 x 2 x 89
+// p = 151 0.094 and 0.034, 673 x 4 x 34 p = 1798 0.157 and 0.057, 2000 x 60 x 500
+// p = 256 0.088 and 0.057).  Wider ones take all: leaving out the last tile's gave
+// 1531 x 1093 x 1777 p = 512 1.13 for 1.14, but 64 uneven products 8.02 for 7.87.
+constexpr int kNarrow = 128;
 template <int NC>
 __device__ __forceinline__ void epi_job(const Job& j, const EpiConst& e, uint32_t tbase, UStage& us) {
   static_assert(NC % 2 == 0, "chunks go in pairs");
+  const int nc = e.N <= kNarrow ? min(NC, (e.N - e.col0 + 31) >> 5) : NC;
+  if (nc <= 0) return;
   uint32_t va[32], vb[32];
   tc::tmem_ld32_nowait(tbase, va);
   tc::tmem_ld_wait_regs(va);
 #pragma unroll 1
-  for (int c = 0; c < NC; c += 2) {
+  for (int c = 0; c < nc; c += 2) {
     tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * (c + 1)), vb);
     epi_chunk(j, e, va, tbase + (uint32_t)(32 * c), 32 * c, us);
     tc::tmem_ld_wait_regs(vb);
-    if (c + 2 < NC) tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * (c + 2)), va);
-    epi_chunk(j, e, vb, tbase + (uint32_t)(32 * (c + 1)), 32 * (c + 1), us);
-    if (c + 2 < NC) tc::tmem_ld_wait_regs(va);
+    if (c + 2 < nc) tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * (c + 2)), va);
+    if (c + 1 < nc) epi_chunk(j, e, vb, tbase + (uint32_t)(32 * (c + 1)), 32 * (c + 1), us);
+    if (c + 2 < nc) tc::tmem_ld_wait_regs(va);
   }
   if (!j.last) tc::tmem_wait_st();
 }

@@ -59,6 +59,27 @@ def test_ragged_rows_match_the_aligned_store(ozk, M, N, K, p, tile):
         assert torch.equal(got, want)
 
 
+@pytest.mark.parametrize("tile", [1, 2])
+@pytest.mark.parametrize("M,K", [(31, 1100), (300, 40)])
+@pytest.mark.parametrize("N", [1, 2, 32, 33, 64, 65, 96, 97, 127, 128])
+def test_narrow_outputs_match_the_wide_ones(ozk, M, N, K, tile):
+    """Up to 128 columns the epilogue takes the chunks that hold any; with zero columns
+    appended up to 256 it takes them all."""
+    rng = np.random.Generator(np.random.PCG64(M * 1000 + N))
+    A, B = synth.mp_matrix(rng, M, K, 200, -8, 8), synth.mp_matrix(rng, K, N, 200, -8, 8)
+    Ad, out = ozk.MPMatrix.from_host(A), []
+    for cols, Bh in ((N, B), (256, _padded(B, 256))):
+        plan = ozk.Plan((M, cols, K, 200), gemm_tile=tile)
+        ws = plan.workspace()
+        ws.fill_(0x5A)
+        C = ozk.MPMatrix.empty(M, cols, 200)
+        plan.execute(Ad, ozk.MPMatrix.from_host(Bh), C, ws)
+        plan.check()
+        out.append((_v(plan, ws, M, cols)[:, :, :N], C.limbs[:, :, :N], C.exp[:, :N], C.sign[:, :N]))
+    for got, want in zip(*out):
+        assert torch.equal(got, want)
+
+
 def test_batch_mixes_both_stores(ozk):
     """Problems with and without TMA-storable rows alternate on the same warps'
     staging buffers; each equals its own single product."""
