@@ -249,6 +249,7 @@ struct DevState {
   ListRef tct[9];               // tensor-core CRT tile lists (smem = kpad_max, lmax = L max)
   int tct_npad[9] = {0};
   ListRef cmt;                  // tensor-core CRT sums: runs of tiles (smem = most formed columns, lmax = most K blocks)
+  const int32_t* cmt_run = nullptr;   // the run of each of their tiles (null: long runs)
   ListRef finl;                 // finish blocks of long accumulators (smem = D max, lmax = output limbs max)
   ListRef fsh[9];               // finish blocks of one-lane classes after the tensor-core sums
   std::vector<ListRef> rmt;     // warp-specialised tensor-core residue tiles, one list per TMEM layout (smem = cw)
@@ -877,7 +878,7 @@ struct TableImage {
   std::vector<size_t> o_tctab;
   // tensor-core CRT sums: runs of tiles; warp-specialised tensor-core residue
   // tiles: one launch per TMEM layout, {first tile, tiles, chunk width}
-  size_t o_cmt = 0, o_finl = 0;
+  size_t o_cmt = 0, o_cmr = 0, o_finl = 0;          // o_cmr 0: long runs
   int n_cmt = 0, cmt_cols = 0, cmt_kb = 0;
   std::vector<std::array<int, 3>> rmt_seg;
   size_t o_fsh[9] = {0};            // short finish blocks per one-lane class (after the tensor-core sums)
@@ -1070,6 +1071,7 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
   // one launch share the column map of their buffers and slots)
   std::map<std::array<int, 3>, std::vector<int4>> rmt_by;
   std::vector<int4> cmt;
+  std::vector<int32_t> cmr;
   for (int pi = 0; pi < count; ++pi) {
     const ProbHost& h = pl->probs[pi];
     const bool own_planes = !h.sum_of;             // planes made by the scan and residue kernels
@@ -1130,6 +1132,7 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
       if (nt > INT_MAX) return OZ2_ERANGE;
       if (nt > INT_MAX - ti.n_cmt) return OZ2_ERANGE;
       cmt.push_back(make_int4(pi, ti.n_cmt, ti.n_cmt + (int)nt, 0));
+      if (count > 1) cmr.insert(cmr.end(), (size_t)nt, (int32_t)cmt.size() - 1);
       ti.n_cmt += (int)nt;
       ti.cmt_cols = std::max(ti.cmt_cols, 32 * h.crt_ngrp);
       ti.cmt_kb = std::max(ti.cmt_kb, h.crt_kpad / 64);
@@ -1212,6 +1215,8 @@ static int build_table_image(ozaki2_plan_s* pl, int sms, TableImage& ti) {
   if (!finl.empty() && crt_finish_long_smem(ti.finl_dmax, ti.finl_nlmax) > 200 * 1024)
     return OZ2_EINTERNAL;
   ti.o_cmt = ti.b.add(cmt.data(), cmt.size() * 16);
+  // a block's next tile is as many tiles on as there are SMs
+  if (cmt.size() > 1 && (int64_t)cmt.size() * sms > ti.n_cmt) ti.o_cmr = ti.b.add(cmr.data(), cmr.size() * 4);
   for (int c = 0; c < 9; ++c) {
     ti.o_fsh[c] = ti.b.add(fsh[c].data(), fsh[c].size() * 16);
     ti.n_fsh[c] = (int)fsh[c].size();
@@ -1271,6 +1276,7 @@ static void install_table_image(ozaki2_plan_s* pl, const TableImage& ti, uint8_t
     d.tct_npad[i] = ti.tct_npad[i];
   }
   d.cmt = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_cmt), ti.n_cmt, ti.cmt_cols, ti.cmt_kb};
+  d.cmt_run = ti.o_cmr ? reinterpret_cast<const int32_t*>(base + ti.o_cmr) : nullptr;
   d.finl = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_finl), ti.n_finl, ti.finl_dmax, ti.finl_nlmax};
   for (int c = 0; c < 9; ++c) d.fsh[c] = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_fsh[c]), ti.n_fsh[c], 0, 0};
   d.rtt = ListRef{reinterpret_cast<const int32_t*>(base + ti.o_rtt), ti.n_rtt, ti.rtt_kpad, ti.rtt_l, ti.na_rtt};
@@ -1642,7 +1648,7 @@ static int enqueue(ozaki2_plan_s* pl, LaunchBlock& lb, uint8_t* ws, cudaStream_t
     OZ2_CU(launch_combine_complex(tab, (int64_t)h.L * (int64_t)(align_up((size_t)(h.M * h.N), 8) / 8), s));
   }
   if (timing) OZ2_CU(cudaEventRecord(pl->ev[3], s));
-  if (d.cmt.n) OZ2_CU(launch_crt_mm(tab, d.cmt.ptr, d.cmt.n, d.cmt.smem, d.cmt.lmax, d.sms, s));
+  if (d.cmt.n) OZ2_CU(launch_crt_mm(tab, d.cmt.ptr, d.cmt_run, d.cmt.n, d.cmt.smem, d.cmt.lmax, d.sms, s));
   if (timing) OZ2_CU(cudaEventRecord(pl->ev[5], s));
   for (int c = 0; c < 9; ++c)
     if (d.fsh[c].n) OZ2_CU(launch_crt_fin_short(tab, c, d.fsh[c].ptr, d.fsh[c].n, s));

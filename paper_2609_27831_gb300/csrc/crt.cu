@@ -1388,7 +1388,7 @@ __global__ void __launch_bounds__(kFinThreads, (ND <= 24 ? 6 : 1)) k_crt_fin_sho
 //                of the pieces of floor(2^28 / m_l): the quotient estimate
 //                alpha~ = floor(sum_l v_l floor(2^28 / m_l) / 2^28), in
 //                {alpha - 1, alpha}, written per output for the finish.
-// Runs of tiles: {problem, first tile, end, 0}.
+// Runs of tiles: {problem, first tile, end, 0}; the run of each tile where they are short.
 // ---------------------------------------------------------------------------
 constexpr int kCmBuildWarps = 8, kCmEpiWarps = 16;
 constexpr int kCmThreads = 32 * (3 + kCmBuildWarps + kCmEpiWarps);
@@ -1416,21 +1416,23 @@ struct CmLayout {
 };
 
 // A run of a problem's tiles in the launch; every role walks the runs on its own.
+// Where runs are shorter than a block's step, run_of holds each tile's; else it is
+// null and the next runs are read in turn.  Sums of 4096 products of 16 x 16 x 16 at
+// p = 300, two tiles each, ms: 0.51 in turn and 0.13 looked up; of 200 of 300 x 200 x
+// 64 at p = 512, 469 tiles each: 1.46 and 1.49.
 struct CmWalk {
-  const int4* seg;
-  int prob, first, end;
-  __device__ CmWalk(const int4* s) : seg(s - 1), prob(-1), first(0), end(0) {}
-  __device__ bool seek(int i) {                      // to the run of tile i; true if it is another one
-    bool moved = false;
+  const int4* segs;
+  const int32_t* run_of;
+  int at, prob, first, end;
+  __device__ CmWalk(const int4* s, const int32_t* r) : segs(s), run_of(r), at(-1), prob(-1), first(0), end(0) {}
+  __device__ void seek(int i) {                      // to the run of tile i
     while (i >= end) {
-      ++seg;
-      const int4 a = __ldg(seg);
+      at = run_of ? __ldg(run_of + i) : at + 1;
+      const int4 a = __ldg(segs + at);
       prob = a.x;
       first = a.y;
       end = a.z;
-      moved = true;
     }
-    return moved;
   }
 };
 
@@ -1479,8 +1481,8 @@ __device__ __forceinline__ void crt_group_small(const uint32_t* y, uint64_t (&ac
 }
 
 __global__ void __launch_bounds__(kCmThreads, 1)
-    k_crt_mm(const __grid_constant__ DevTables T, const int4* __restrict__ segs, int ntiles, uint32_t stage_bytes,
-             int stages, int uslots, int cmax) {
+    k_crt_mm(const __grid_constant__ DevTables T, const int4* __restrict__ segs, const int32_t* __restrict__ run_of,
+             int ntiles, uint32_t stage_bytes, int stages, int uslots, int cmax) {
   using namespace tc;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -1550,7 +1552,7 @@ __global__ void __launch_bounds__(kCmThreads, 1)
       int issued_phase[kCmMaxStages];
       for (int i = 0; i < kCmMaxStages; ++i) issued_phase[i] = -1;
       bool ok = true;
-      CmWalk walk(segs);
+      CmWalk walk(segs, run_of);
       for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
         walk.seek(i);
         if (walk.prob == prev && nkb <= stages) continue;     // this problem's table is in the ring
@@ -1591,7 +1593,7 @@ __global__ void __launch_bounds__(kCmThreads, 1)
       auto wait = [&](uint64_t* bar, uint32_t parity) {
         return ok = mbar_wait_warp(bar, parity, abort_flag, T.status, T.spin_limit);
       };
-      CmWalk walk(segs);
+      CmWalk walk(segs, run_of);
       for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x, ++t) {
         walk.seek(i);
         const bool fresh = !stay || walk.prob != prev;          // the table's stages are waited for
@@ -1658,7 +1660,7 @@ __global__ void __launch_bounds__(kCmThreads, 1)
       int issued_phase[kCmMaxUSlots];
       for (int i = 0; i < kCmMaxUSlots; ++i) issued_phase[i] = -1;
       bool ok = true;
-      CmWalk walk(segs);
+      CmWalk walk(segs, run_of);
       for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
         walk.seek(i);
         if (walk.prob != prev) {
@@ -1691,7 +1693,7 @@ __global__ void __launch_bounds__(kCmThreads, 1)
     int us = 0, vs = 0, L = 0, prev = -1;
     uint32_t uph = 0, vph = 1;                        // vph: parity of the block's last release
     bool ok = true, first_round = true;
-    CmWalk walk(segs);
+    CmWalk walk(segs, run_of);
     for (int i = blockIdx.x; ok && i < ntiles; i += gridDim.x) {
       walk.seek(i);
       if (walk.prob != prev) {
@@ -1734,7 +1736,7 @@ __global__ void __launch_bounds__(kCmThreads, 1)
     bool ok = true, small = false;
     int64_t up = 0, mn = 0;
     uint32_t *qbase = nullptr, *abase = nullptr;
-    CmWalk walk(segs);
+    CmWalk walk(segs, run_of);
     for (int i = blockIdx.x; i < ntiles; i += gridDim.x, ++t) {
       walk.seek(i);
       if (walk.prob != prev) {
@@ -1899,15 +1901,15 @@ static int crt_mm_uslots(int cmax, int stages) {
 }
 bool crt_mm_fits(int cols) { return cols <= kCmCols && crt_mm_stages(cols, kCmMaxStages) >= 2; }
 
-cudaError_t launch_crt_mm(const DevTables& t, const int32_t* segs, int ntiles, int cmax, int kbmax, int sms,
-                          cudaStream_t s) {
+cudaError_t launch_crt_mm(const DevTables& t, const int32_t* segs, const int32_t* run_of, int ntiles, int cmax,
+                          int kbmax, int sms, cudaStream_t s) {
   if (ntiles == 0) return cudaSuccess;
   const int stages = crt_mm_stages(cmax, kbmax);
   if (stages == 0) return cudaErrorInvalidValue;
   const int us = crt_mm_uslots(cmax, stages);
   const uint32_t stage_bytes = (uint32_t)cmax * 128u;
   k_crt_mm<<<ntiles < sms ? ntiles : sms, kCmThreads, CmLayout(stage_bytes, stages, us).total, s>>>(
-      t, reinterpret_cast<const int4*>(segs), ntiles, stage_bytes, stages, us, cmax);
+      t, reinterpret_cast<const int4*>(segs), run_of, ntiles, stage_bytes, stages, us, cmax);
   return cudaGetLastError();
 }
 

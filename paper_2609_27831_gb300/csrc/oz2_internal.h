@@ -189,11 +189,11 @@ cudaError_t launch_crt_tc(const DevTables& t, int cls, const int32_t* tiles, int
                           int npad_max, int lmax, int sms, cudaStream_t s);
 int crt_tc_smem_bytes(int cls, int kpad_max, int npad_max, int lmax, int nbuf);
 // Tensor-core CRT sums of any length (crt_mode 2): runs of tiles of 128 outputs
-// {problem, first tile, end, 0}, cmax and kbmax the most formed columns and K
-// blocks of 64; group sums to the workspace.  Then the finish of long accumulators, blocks of 128
+// {problem, first tile, end, 0} and, where they are short, the run of each tile (else null),
+// cmax and kbmax the most formed columns and K blocks of 64; group sums to the workspace.  Then the finish of long accumulators, blocks of 128
 // outputs {problem, block}.
-cudaError_t launch_crt_mm(const DevTables& t, const int32_t* segs, int ntiles, int cmax, int kbmax, int sms,
-                          cudaStream_t s);
+cudaError_t launch_crt_mm(const DevTables& t, const int32_t* segs, const int32_t* run_of, int ntiles, int cmax,
+                          int kbmax, int sms, cudaStream_t s);
 bool crt_mm_fits(int cols);
 // the finish of one-lane classes after the tensor-core sums (the host uses it up to 24 digits)
 cudaError_t launch_crt_fin_short(const DevTables& t, int cls, const int32_t* blk, int nblk, cudaStream_t s);

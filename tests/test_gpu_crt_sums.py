@@ -70,6 +70,22 @@ def test_several_tiles_per_block(ozk, p):
     assert _same(*out)
 
 
+def test_many_short_runs(ozk):
+    """More problems than SMs, of one tile to three: a block's next tile lies many runs ahead."""
+    ps = (113, 256, 300, 512, 700)
+    shapes = [((16, 8), (13, 11), (17, 17))[i % 3] + (4, ps[i % 5]) for i in range(400)]
+    triples, singles = [], []
+    for i, (M, N, K, p) in enumerate(shapes):
+        A, B = _operands(ozk, M, N, K, p, i)
+        triples.append((A, B, ozk.MPMatrix.empty(M, N, p)))
+        singles.append(ozk.gemm(A, B, crt_engine=3))
+    plan = ozk.Plan(shapes, crt_engine=2)
+    plan.execute_batched(triples, plan.workspace())
+    plan.check()
+    for (_, _, C), S in zip(triples, singles):
+        assert _same(C, S)
+
+
 def test_batch_mixes_tables(ozk):
     """Runs of tiles of different problems on one block: resident and streamed tables, one and two
     column chunks in a launch sized by the longest, a run shorter than the grid."""
