@@ -787,15 +787,19 @@ static void layout_workspace(ozaki2_plan_s* pl) {
 
 // Automatic plane GEMM tile: CTA pairs (256 x 256) where they cover the outputs with
 // at most 12 % more tile area (weighted by K) than 128 x 256 tiles, where the plane
-// products fill the 152 SMs at least four times over, and below 1e13 flop.  Measured
+// products fill the 152 SMs at least four times over, and where no product has 1e13
+// flop or more.  Measured
 // on one GB300, one SM and pairs, plane GEMM stage in ms: 1024^3 p = 256 0.156 and
 // 0.137, 1531 x 1093 x 1777 p = 512 1.50 and 1.15, 64 uneven products (1.08 times
 // the area) 8.49 and 7.89; equal at 2.8 to 5.4 rounds (256^3 p = 512, 512^3 p = 256);
 // below, 384^3 p = 53 0.0143 and 0.0185, and with 20 % more area 611 x 347 x 923
-// p = 113 0.039 and 0.045.  Beyond 1e13 flop the power cap evens them out: 8192^3
-// p = 53 20.1 and 20.0 ms for the product, 4096^3 p = 2048 113.2 and 115.0.
+// p = 113 0.039 and 0.045.  Beyond 1e13 flop the power cap evens out the largest: 8192^3
+// p = 53 20.1 and 20.0 ms for the product, 4096^3 p = 2048 113.2 and 115.0 (not every
+// one: 3000^3 p = 512 18.2 and 13.8).  The limit is each product's, not the plan's:
+// complex 3000^3 p = 256, three of 5.5e12, 27.0 and 21.0 ms, 4096^3 p = 113 15.5 and
+// 14.3; batches of eight 2048^3 p = 256 16.7 and 16.0, of four 3000^3 36.8 and 28.4.
 struct TileLoad {
-  double rounds = 0, one = 0, two = 0, flops = 0;
+  double rounds = 0, one = 0, two = 0, flops = 0;   // flops: of the largest product
   // a product's planes G from the modulus rule (Eq. 3 and Eq. crtcond), without building it
   void add(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts& o, const PlanExtra& ex = PlanExtra()) {
     if (M <= 0 || N <= 0 || K <= 0 || M > INT_MAX || N > INT_MAX || K > kMaxK || p < 2 || p > kMaxP) return;
@@ -809,7 +813,7 @@ struct TileLoad {
     const double n1 = G * (double)((M + 127) / 128) * (double)((N + 255) / 256);
     const double n2 = G * (double)((M + 255) / 256) * (double)((N + 255) / 256);
     rounds += n1 / 152;
-    flops += 2.0 * G * (double)M * (double)N * (double)K;
+    flops = std::max(flops, 2.0 * G * (double)M * (double)N * (double)K);
     one += n1 * (double)K;
     two += 2 * n2 * (double)K;
   }

@@ -184,6 +184,17 @@ def test_residue_engine_choice(ozk):
     assert ozk.Plan((64, 64, 64, 256), res_engine=2).info["res_mode"] == 2
 
 
+def test_the_tile_limit_is_each_product_s(ozk):
+    """CTA pairs up to 1e13 plane flops of one product (5.5e12 at 3000^3, p = 256), however
+    many the plan has: a complex one has three."""
+    one, over = (3000, 3000, 3000, 256), (4096, 4096, 4096, 2048)
+    assert ozk.Plan(one).info["gemm_tile"] == 2
+    assert ozk.ComplexPlan(one).info["gemm_tile"] == 2
+    assert ozk.Plan([one] * 4).info["gemm_tile"] == 2
+    assert ozk.Plan(over).info["gemm_tile"] == 1
+    assert ozk.Plan([(1024, 1024, 1024, 256), over]).info["gemm_tile"] == 1
+
+
 def test_planes_streamed_in_modulus_groups(ozk):
     """Large products stream their residue planes through the workspace in
     groups of consecutive moduli: one group's bf16 plane stacks at a time
