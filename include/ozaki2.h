@@ -96,7 +96,8 @@ typedef struct {
   int engine;     /* OZ2_ENGINE_* */
   int k_chunk;    /* K per exact fp32 accumulation chunk: multiple of 64, <= 1024;
                      0 = 1024 (127^2 * 1024 + 16191 < 2^24 keeps every partial sum exact) */
-  int grid;       /* persistent CTAs of the grouped GEMM; 0 = one per SM */
+  int grid;       /* most persistent CTAs of the grouped GEMM; 0 = one per SM (gemm_tile 2 with
+                     an odd number runs one less, with 1 two) */
   int schedule;   /* OZ2_SCHED_* */
   int timing;     /* nonzero: record per-stage CUDA events (ozaki2_last_timings) */
   int crt_engine; /* 0: automatic (default): engine 2 where the CRT accumulator needs more than

@@ -785,9 +785,11 @@ static void layout_workspace(ozaki2_plan_s* pl) {
   pl->ws_bytes = off;
 }
 
+constexpr int kTileSMs = 152;      // SMs that the tile rule counts on (a plan is made without a device)
+
 // Automatic plane GEMM tile: CTA pairs (256 x 256) where they cover the outputs with
 // at most 12 % more tile area (weighted by K) than 128 x 256 tiles, where the plane
-// products fill the 152 SMs at least four times over, and where no product has 1e13
+// products fill the SMs at least four times over, and where no product has 1e13
 // flop or more.  Measured
 // on one GB300, one SM and pairs, plane GEMM stage in ms: 1024^3 p = 256 0.156 and
 // 0.137, 1531 x 1093 x 1777 p = 512 1.50 and 1.15, 64 uneven products (1.08 times
@@ -798,8 +800,12 @@ static void layout_workspace(ozaki2_plan_s* pl) {
 // one: 3000^3 p = 512 18.2 and 13.8).  The limit is each product's, not the plan's:
 // complex 3000^3 p = 256, three of 5.5e12, 27.0 and 21.0 ms, 4096^3 p = 113 15.5 and
 // 14.3; batches of eight 2048^3 p = 256 16.7 and 16.0, of four 3000^3 36.8 and 28.4.
+// A plan with a bound on its CTAs (opts.grid) takes pairs where they are as many: at an
+// even bound.
 struct TileLoad {
+  int grid;                                         // CTAs that the plan may use
   double rounds = 0, one = 0, two = 0, flops = 0;   // flops: of the largest product
+  explicit TileLoad(const ozaki2_opts& o) : grid(o.grid > 0 ? o.grid : kTileSMs) {}
   // a product's planes G from the modulus rule (Eq. 3 and Eq. crtcond), without building it
   void add(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts& o, const PlanExtra& ex = PlanExtra()) {
     if (M <= 0 || N <= 0 || K <= 0 || M > INT_MAX || N > INT_MAX || K > kMaxK || p < 2 || p > kMaxP) return;
@@ -812,12 +818,12 @@ struct TileLoad {
     const double G = L1 + 3.0 * (L - L1);
     const double n1 = G * (double)((M + 127) / 128) * (double)((N + 255) / 256);
     const double n2 = G * (double)((M + 255) / 256) * (double)((N + 255) / 256);
-    rounds += n1 / 152;
+    rounds += n1 / grid;
     flops = std::max(flops, 2.0 * G * (double)M * (double)N * (double)K);
     one += n1 * (double)K;
     two += 2 * n2 * (double)K;
   }
-  bool pairs() const { return rounds >= 4 && two <= 1.12 * one && flops < 1e13; }
+  bool pairs() const { return grid % 2 == 0 && rounds >= 4 && two <= 1.12 * one && flops < 1e13; }
 };
 static bool auto_tile(const ozaki2_plan_s* pl) { return pl->opts.gemm_tile == 0 && pl->opts.engine == OZ2_ENGINE_TC; }
 
@@ -835,7 +841,7 @@ static int new_plan(const ozaki2_opts* opts, ozaki2_plan_s** res) {
     delete pl;
     return OZ2_EINVAL;
   }
-  pl->tile2 = o.engine == OZ2_ENGINE_TC && o.gemm_tile == 2;   // automatic: decided per plan (plan_tile)
+  pl->tile2 = o.engine == OZ2_ENGINE_TC && o.gemm_tile == 2;   // automatic: decided where the plan is built (TileLoad)
   *res = pl;
   return OZ2_OK;
 }
@@ -1714,7 +1720,7 @@ int plan_create_ex(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts* op
   pl->no_stream = true;                          // the binary64 mode keeps every plane for the backward
   try {
     if (auto_tile(pl)) {
-      TileLoad tl;
+      TileLoad tl(pl->opts);
       tl.add(M, N, K, p, pl->opts, ex);
       pl->tile2 = tl.pairs();
     }
@@ -1797,7 +1803,7 @@ int ozaki2_plan_create(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts
   if (rc) return rc;
   try {
     if (auto_tile(pl)) {
-      TileLoad tl;
+      TileLoad tl(pl->opts);
       tl.add(M, N, K, p, pl->opts);
       pl->tile2 = tl.pairs();
     }
@@ -1843,7 +1849,7 @@ int ozaki2_plan_create_batched_ex(int count, const ozaki2_problem* shapes, const
   }
   try {
     if (auto_tile(pl)) {
-      TileLoad tl;
+      TileLoad tl(pl->opts);
       for (int i = 0; i < count; ++i)
         tl.add(shapes[i].M, shapes[i].N, shapes[i].K, shapes[i].p, po.empty() ? pl->opts : po[i]);
       pl->tile2 = tl.pairs();
@@ -1870,7 +1876,7 @@ int ozaki2_plan_create_complex(int64_t M, int64_t N, int64_t K, int p, const oza
   ex.inner = 2 * K;                              // |Cr_hat|, |Ci_hat| <= 2K 2^(2t)
   try {
     if (auto_tile(pl)) {
-      TileLoad tl;
+      TileLoad tl(pl->opts);
       for (int i = 0; i < 3; ++i) tl.add(M, N, K, p, pl->opts, ex);
       pl->tile2 = tl.pairs();
     }

@@ -195,6 +195,16 @@ def test_the_tile_limit_is_each_product_s(ozk):
     assert ozk.Plan([(1024, 1024, 1024, 256), over]).info["gemm_tile"] == 1
 
 
+@pytest.mark.parametrize("grid,tile", [(0, 2), (1, 1), (2, 2), (7, 1), (64, 2), (151, 1), (152, 2)])
+def test_automatic_pairs_keep_to_the_grid(ozk, grid, tile):
+    """opts.grid bounds the CTAs: a pair is two of them, so the automatic choice takes pairs
+    at an even bound only (a grid of one ran two CTAs, one of seven ran six)."""
+    one = (1024, 1024, 1024, 256)
+    assert ozk.Plan(one, grid=grid).info["gemm_tile"] == tile
+    assert ozk.Plan([one, (512, 512, 64, 256)], grid=grid).info["gemm_tile"] == tile
+    assert ozk.ComplexPlan(one, grid=grid).info["gemm_tile"] == tile
+
+
 def test_planes_streamed_in_modulus_groups(ozk):
     """Large products stream their residue planes through the workspace in
     groups of consecutive moduli: one group's bf16 plane stacks at a time
