@@ -262,6 +262,18 @@ def test_plane_group_option_errors(ozk):
         assert ozk.Plan((200, 150, 300, 256), **kw).info["plane_groups"] == 1
 
 
+@pytest.mark.parametrize("t", [2113, 10 ** 8, 2 ** 30, 2 ** 31 - 1])
+def test_widths_beyond_every_modulus_set_are_refused(ozk, t):
+    """At once, whatever the plan's kind: the tile rule formed the bound's 2 t + 2 bits (an
+    exception out of the C entry from t = 2^30 on)."""
+    shape = (1024, 1024, 64, 53)
+    for make in (lambda: ozk.Plan(shape, t_bits=t), lambda: ozk.Plan([shape] * 2, t_bits=t),
+                 lambda: ozk.ComplexPlan(shape, t_bits=t)):
+        with pytest.raises(ozk.OzakiError) as ei:
+            make()
+        assert ei.value.status == ozk._lib.OZ2_ERANGE
+
+
 @pytest.mark.parametrize("keep", [True, False])
 def test_refused_binary64_forwards_allocate_nothing(ozk, keep):
     """A null operand or a short stride is refused on the host: OZ2_EINVAL for
