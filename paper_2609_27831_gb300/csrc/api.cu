@@ -339,6 +339,12 @@ cudaError_t init_crt_attributes();
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// The internal width t of a problem (Eq. 3), whatever the sum of the caller's values.
+static int64_t internal_bits(int64_t inner, int p, const ozaki2_opts& o, const PlanExtra& ex) {
+  if (ex.force_t > 0) return ex.force_t;
+  return o.t_bits > 0 ? o.t_bits : (int64_t)p + o.guard_bits + ceil_log2(inner);
+}
+
 // The shortest prefix of the modulus list with P > inner 2^(2t + 2) (Eq.
 // crtcond with the implementation's +2 margin, Sec. 4.3), or exactly force_L
 // moduli when force_L > 0 (which must still meet the bound); its length, or
@@ -454,9 +460,9 @@ static int build_problem(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int
   h.M = M; h.N = N; h.K = K; h.p = p;
   h.nl = (p + 63) / 64;
   const int64_t inner = std::max<int64_t>(K, ex->inner);
-  h.t = ex->force_t > 0 ? ex->force_t
-                        : (o.t_bits > 0 ? o.t_bits : p + o.guard_bits + ceil_log2(inner));   // Eq. 3
-  if (h.t > kMaxP + 64) return OZ2_ERANGE;
+  const int64_t t = internal_bits(inner, p, o, *ex);
+  if (t > kMaxP + 64) return OZ2_ERANGE;
+  h.t = (int)t;
   Big P;
   const int L = modulus_prefix(inner, h.t, ex->force_L, &P);
   if (L < 0) return OZ2_ERANGE;
@@ -789,14 +795,14 @@ static void layout_workspace(ozaki2_plan_s* pl) {
 // where P and the bound agree to 13 digits.  (By big integers, as the plan itself does
 // it, the rule cost half as much again: a batch of 4096 products 8.9 ms to plan
 // without it, 13.5 with, 9.3 so.)
-static int modulus_prefix_estimate(int64_t inner, int t) {
+static int modulus_prefix_estimate(int64_t inner, int64_t t) {
   static const std::vector<double> bits = [] {
     std::vector<double> v;
     double s = 0;
     for (int m : modulus_list()) v.push_back(s += std::log2((double)m));
     return v;
   }();
-  const auto it = std::upper_bound(bits.begin(), bits.end(), std::log2((double)inner) + 2.0 * t + 2);
+  const auto it = std::upper_bound(bits.begin(), bits.end(), std::log2((double)inner) + 2.0 * (double)t + 2);
   return it == bits.end() ? -1 : (int)(it - bits.begin()) + 1;
 }
 
@@ -825,7 +831,7 @@ struct TileLoad {
   void add(int64_t M, int64_t N, int64_t K, int p, const ozaki2_opts& o, const PlanExtra& ex = PlanExtra()) {
     if (M <= 0 || N <= 0 || K <= 0 || M > INT_MAX || N > INT_MAX || K > kMaxK || p < 2 || p > kMaxP) return;
     const int64_t inner = std::max<int64_t>(K, ex.inner);
-    const int t = ex.force_t > 0 ? ex.force_t : (o.t_bits > 0 ? o.t_bits : p + o.guard_bits + ceil_log2(inner));
+    const int64_t t = internal_bits(inner, p, o, ex);
     const int L = ex.force_L > 0 ? ex.force_L : modulus_prefix_estimate(inner, t);
     if (L < 0) return;
     const int L1 = std::min(L, one_limb_count());

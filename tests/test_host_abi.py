@@ -274,6 +274,17 @@ def test_widths_beyond_every_modulus_set_are_refused(ozk, t):
         assert ei.value.status == ozk._lib.OZ2_ERANGE
 
 
+@pytest.mark.parametrize("g", [2 ** 30, 2 ** 31 - 60, 2 ** 31 - 1])
+def test_guard_bits_do_not_wrap(ozk, g):
+    """p + guard_bits + ceil(log2 K) beyond an int is out of range, not a negative width."""
+    shape = (1024, 1024, 64, 53)
+    for make in (lambda: ozk.Plan(shape, guard_bits=g), lambda: ozk.Plan([shape] * 2, guard_bits=g),
+                 lambda: ozk.ComplexPlan(shape, guard_bits=g)):
+        with pytest.raises(ozk.OzakiError) as ei:
+            make()
+        assert ei.value.status == ozk._lib.OZ2_ERANGE
+
+
 @pytest.mark.parametrize("keep", [True, False])
 def test_refused_binary64_forwards_allocate_nothing(ozk, keep):
     """A null operand or a short stride is refused on the host: OZ2_EINVAL for
