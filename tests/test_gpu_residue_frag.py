@@ -56,6 +56,41 @@ def test_planes_match_the_byte_gemm(ozk, M, N, K, p, t):
     assert torch.equal(C.limbs, D.limbs) and torch.equal(C.exp, D.exp) and torch.equal(C.sign, D.sign)
 
 
+@pytest.mark.parametrize("t", [63, 127, 191, 319, 575])
+def test_the_largest_byte_sums(ozk, t):
+    """Integers of ones, +-(2^t - 1): every byte 255 (the top one 127 at whole bytes less a bit), the
+    sums at their bounds; each plane against the residue itself."""
+    M, N, K, p = 9, 10, 40, t
+    nl = (p + 63) // 64
+    rng = np.random.Generator(np.random.PCG64(t))
+
+    def ones(rows, cols):
+        limbs = np.full((nl, rows, cols), 2 ** 64 - 1, dtype=np.uint64)
+        limbs[0] = np.uint64((2 ** 64 - 1) ^ ((1 << (64 * nl - p)) - 1))
+        return {"p": p, "limbs": limbs, "exp": np.zeros((rows, cols), np.int32),
+                "sign": rng.integers(0, 2, (rows, cols)).astype(np.int8)}
+
+    A, B = ones(M, K), ones(K, N)
+    mode, pa, pb, _ = _planes(ozk, ozk.MPMatrix.from_host(A), ozk.MPMatrix.from_host(B), (M, N, K, p), 0x5A, t_bits=t)
+    assert mode == 0
+    mods = ozk.Plan((M, N, K, p), t_bits=t).moduli()
+    for planes, sign in ((pa, A["sign"]), (pb, B["sign"].T)):
+        v = planes.cpu().view(torch.bfloat16).to(torch.int64).numpy()
+        s = np.where(sign != 0, -1, 1)
+        at = 0
+        for m in mods:
+            r = pow(2, t, m) - 1
+            if m <= 255:
+                x, at = v[at], at + 1
+            else:
+                r0, r1, rs = v[at:at + 3]
+                assert np.array_equal(rs, r0 + r1) and r0.min() > -64 and r0.max() <= 64
+                x, at = r0 + 128 * r1, at + 3
+            assert np.array_equal(np.mod(x, m), np.mod(s * r, m)), m
+            assert 2 * x.max() <= m and 2 * x.min() > -m, m
+        assert at == v.shape[0]
+
+
 @pytest.mark.parametrize("gmax", [20, 61])
 def test_groups_of_moduli(ozk, gmax):
     """Planes streamed in groups: fewer moduli and tiles per launch, with and without the even one."""

@@ -1,12 +1,13 @@
 """Arithmetic facts the CUDA kernels rely on, checked exhaustively on the CPU.
 
-The CUDA-core residue kernel reduces the byte-product sum a (one-limb
-modulus m, a <= 4 * 32 words * 255 * 250 < 2^23) in fp32 with
-q = round(a * rcp), rcp = 1/m rounded to fp32 as the library's host code
-computes it.  For odd m the kernel takes r = a - q m as the centered residue
-without a correction step; that holds exactly when q = round(a / m) for every
-such a, which this test checks for all odd one-limb moduli of the method
-(Sec. 4.3's moduli <= 255) and every reachable a.
+The residue kernel for integers of up to 72 bytes reduces the signed byte-product
+sum y (one-limb modulus m, |y| <= 72 * 255 * 250 < 2^23) in packed fp32 with
+q = round(y * rcp), rcp = 1/m rounded to fp32 as the library's host code
+computes it, and takes r = y - q m as the centered residue without a correction
+step; for odd m that holds exactly when q = round(y / m) for every such y, which
+this test checks for all odd one-limb moduli of the method (Sec. 4.3's moduli
+<= 255) and every reachable |y| (rounding to nearest is odd in y).  (The form for
+longer integers reduces 32-bit sums by Barrett's method and needs none of this.)
 """
 import numpy as np
 
@@ -16,8 +17,8 @@ from oracle import ozaki2_oracle as o
 def test_fp32_rounded_quotient_is_exact_for_odd_one_limb_moduli():
     mods = [m for m in o.Params(1024, 2048).moduli if m <= 255]
     assert len(mods) == 54 and sum(m % 2 == 0 for m in mods) == 1      # 128 is the even one
-    amax = 4 * 32 * 255 * 250
-    assert amax < 2 ** 23
+    amax = 72 * 255 * 250
+    assert amax < 0.973 * 2 ** 23 and 72 * 255 ** 2 < 2 ** 23      # fp32 holds every partial sum
     a = np.arange(amax + 1, dtype=np.int64)
     af = a.astype(np.float64)
     for m in mods:
@@ -35,30 +36,49 @@ def test_fp32_rounded_quotient_is_exact_for_odd_one_limb_moduli():
 
 def test_fp32_rounded_quotient_is_exact_for_two_limb_moduli():
     """Two-limb moduli (odd primes in (255, 16191]): the kernel reduces the
-    high-byte sum with the rounded quotient, then y = s lo + 256 r_hi the same
-    way; up to 24 words |y| <= 24 * 4 * 255^2 + 256 * 8095 < 2^23 / (1 + 2^-29)
-    (beyond, up to 32 words, the low-byte sum is reduced first and |y| < 2^21).
-    Exhaustive over |y| <= 4 * 32 * 255^2 (which covers both) for the smallest,
-    the largest and a spread of the moduli in between."""
+    high-byte sum hi, |hi| <= 72 * 255 * 63, with the rounded quotient, then
+    y = lo + 256 r_hi, |y| <= 72 * 255^2 + 256 * 8095 < 2^23 / (1 + 2^-29), the
+    same way.  Exhaustive over that |y| (the larger range) for the smallest, the
+    largest and a spread of the moduli in between."""
     mods = [m for m in o.Params(1024, 2048).moduli if m > 255]
     assert all(m % 2 == 1 for m in mods)
     pick = sorted(set([mods[0], mods[-1]] + mods[:: max(1, len(mods) // 10)]))
-    amax = 4 * 32 * 255 * 255
+    assert max(mods) <= 16191
+    amax = 72 * 255 * 255 + 256 * 8095
     assert amax * (1 + 2.0 ** -29) < 2 ** 23
-    assert 24 * 4 * 255 * 255 + 256 * 8095 <= amax
+    assert max(m >> 8 for m in mods) == 63 and 72 * 255 * 63 < amax
     a = np.arange(amax + 1, dtype=np.int64)
     af = a.astype(np.float64)
     for m in pick:
         rcp = np.float64(np.float32(1.0 / m))
         q = np.rint(af * rcp).astype(np.int64)
         assert np.array_equal(q, (2 * a + m) // (2 * m)), m
-    # y = r_lo + 256 r_hi over its whole range, for the same moduli
-    for m in pick:
-        h = (m - 1) // 2
-        y = np.arange(-257 * h, 257 * h + 1, dtype=np.int64)
-        rcp = np.float64(np.float32(1.0 / m))
-        q = np.rint(y.astype(np.float64) * rcp).astype(np.int64)
-        assert np.array_equal(q, np.floor_divide(2 * y + m, 2 * m)), m
+
+
+def test_ties_of_the_even_modulus_are_flipped():
+    """m = 128, whose reciprocal and quotients are exact: rounding to nearest even
+    leaves -64 for some multiples of 64, and only there; the kernel flips the sign
+    of that bf16 value (-m/2, bits 0xC280) into +64."""
+    y = np.arange(-72 * 255 * 250, 72 * 255 * 250 + 1, dtype=np.int64)
+    r = y - 128 * np.rint(y / 128.0).astype(np.int64)
+    assert r.min() == -64 and r.max() == 64 and np.all((y[r == -64] & 127) == 64)
+    assert np.float32(-64.0).view(np.uint32) >> 16 == 0xC280
+    flipped = np.where(r == -64, 64, r)
+    assert np.array_equal(np.mod(flipped - y, 128), np.zeros_like(y)) and flipped.min() == -63
+
+
+def test_byte_sums_of_the_crt_stay_exact():
+    """The CRT of up to 12 digits: v_l and the bytes of M_l (and of floor(2^32 / m_l))
+    below 2^8 and at most 48 moduli, so fp32 sums below 48 * 254 * 255 < 2^22; a digit's
+    four byte sums y0 + 2^8 y1 fit 32 bits and lo + 2^16 hi 64, biased by 2^23's bits."""
+    top = 48 * 254 * 255
+    assert top < 2 ** 22
+    bias = (0x4B000000 + (0x4B000000 << 8)) & 0xFFFFFFFF
+    for y0, y1 in ((0, 0), (top, top), (1, top), (top, 0)):
+        bits = [int(np.float32(y + 8388608.0).view(np.uint32)) for y in (y0, y1)]
+        assert bits[0] == 0x4B000000 + y0
+        assert (bits[0] + (bits[1] << 8) - bias) & 0xFFFFFFFF == y0 + (y1 << 8) < 2 ** 32
+    assert sum(m <= 255 for m in o.Params(1024, 2048).moduli) >= 48
 
 
 def test_tensor_core_two_limb_reduction_needs_no_correction():
