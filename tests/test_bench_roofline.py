@@ -26,6 +26,19 @@ def test_cuda_core_crt_stage():
     assert out["gemm"]["achieved"] == pytest.approx(2.0 * M * N * K * 102 / 0.18e-3 / 1e12, rel=1e-3)
 
 
+def test_tensor_stages_are_set_against_the_burst_peak(monkeypatch):
+    peaks = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0, "sm_max_mhz": 2070.0}
+    monkeypatch.setattr(bench, "load_peaks", lambda: (peaks, "measured"))
+    ms = 2.0 * 4096 ** 3 * 879 / 1.85e15 * 1e3               # 1850 TFLOP/s, above the sustained peak
+    st = {"scan": 0.1, "residues": 35.0, "gemm": ms, "crt_sums": 8.0, "crt_finish": 6.0}
+    out = bench.stage_rooflines(_info(G=879, L=329, t=2076, crt_digits=131, crt_pieces=597, res_mode=2), 4096, 4096,
+                                4096, 2048, st, "none")
+    g = out["gemm"]
+    assert g["peak"] == 1900.0 and "burst" in g["peak_source"]
+    assert g["frac"] == pytest.approx(1850 / 1900, abs=1e-3) and g["frac_sustained"] == pytest.approx(1850 / 1700, abs=1e-3)
+    assert all(out[k]["peak"] == 1900.0 for k in ("residues", "crt_sums"))
+
+
 def test_tensor_core_crt_stages():
     M = N = K = 1024
     st = {"scan": 0.02, "residues": 0.2, "gemm": 0.18, "crt_sums": 0.15, "crt_finish": 0.09}
