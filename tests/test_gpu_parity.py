@@ -209,7 +209,7 @@ def test_zero_lines_and_tiny_shapes(ozk):
 def test_p2048_small(ozk):
     """p = 2048 (the largest precision): 32-limb inputs, two-limb moduli; the
     residues and the CRT both on the tensor cores (the defaults at this length)
-    and on the CUDA cores (132-digit residue class, 32-lane CRT groups); every
+    and by engine 3 of each (132-digit dp4a class, 32-lane CRT groups); every
     stage bit-exact."""
     rng = np.random.Generator(np.random.PCG64(2030))
     A = synth.mp_matrix(rng, 20, 24, 2048, -64, 64)
@@ -311,14 +311,15 @@ def test_crt_sum_engine_stages(ozk, shape):
 
 def test_crt_sum_engine_many_tiles(ozk):
     """More 128-output tiles than CTAs (V rebuilt, TMEM slots and rings
-    cycling): identical to the CUDA-core CRT, and sampled entries against the
-    oracle."""
+    cycling): identical to the lane groups' CRT (engine 3), and sampled entries
+    against the oracle."""
     M, N, K, p = 256, 160, 16, 1024
     rng = np.random.Generator(np.random.PCG64(2045))
     A = synth.mp_matrix(rng, M, K, p, -20, 20)
     B = synth.mp_matrix(rng, K, N, p, -20, 20)
     g2 = run_gpu(ozk, A, B, p, debug=False, crt_engine=2)
-    g0 = run_gpu(ozk, A, B, p, debug=False)
+    g0 = run_gpu(ozk, A, B, p, debug=False, crt_engine=3)
+    assert (g2["plan"].info["crt_mode"], g0["plan"].info["crt_mode"]) == (2, 0)
     for key in ("limbs", "exp", "sign"):
         assert np.array_equal(g2["C"][key], g0["C"][key])
     rnd = random.Random(11)
@@ -330,13 +331,14 @@ def test_crt_sum_engine_many_tiles(ozk):
 def test_crt_sum_engine_one_chunk_many_tiles(ozk):
     """One 128-column chunk per tile (p = 256) and many tiles per CTA: the half
     without a chunk in a tile must still wait for that tile's MMAs before it
-    rewrites V.  Identical to the CUDA-core CRT."""
+    rewrites V.  Identical to the CRT of a lane per output (engine 3)."""
     M, N, K, p = 512, 448, 8, 256
     rng = np.random.Generator(np.random.PCG64(2047))
     A = synth.mp_matrix(rng, M, K, p, -20, 20)
     B = synth.mp_matrix(rng, K, N, p, -20, 20)
     g2 = run_gpu(ozk, A, B, p, debug=False, crt_engine=2)
-    g0 = run_gpu(ozk, A, B, p, debug=False)
+    g0 = run_gpu(ozk, A, B, p, debug=False, crt_engine=3)
+    assert (g2["plan"].info["crt_mode"], g0["plan"].info["crt_mode"]) == (2, 0)
     for key in ("limbs", "exp", "sign"):
         assert np.array_equal(g2["C"][key], g0["C"][key])
 
@@ -381,7 +383,7 @@ def test_residue_engines_bit_exact(ozk, shape, engine):
 def test_residue_mm_engine_chunks_and_tiles(ozk, shape):
     """The warp-specialised tensor-core residues with several column chunks
     (p = 1024, 2048), 512 TMEM columns, and more tiles than CTAs (p = 113):
-    planes bit for bit against the CUDA-core kernel and the oracle."""
+    planes bit for bit against the register form and the oracle."""
     M, N, K, p = shape
     rng = np.random.Generator(np.random.PCG64(2050 + p))
     A = synth.zero_rows(synth.mp_matrix(rng, M, K, p, -50, 50), [2])
@@ -391,6 +393,7 @@ def test_residue_mm_engine_chunks_and_tiles(ozk, shape):
     else:
         g2 = run_gpu(ozk, A, B, p, debug=False, res_engine=2)
         g0 = run_gpu(ozk, A, B, p, debug=False)
+        assert (g2["plan"].info["res_mode"], g0["plan"].info["res_mode"]) == (2, 0)
         assert np.array_equal(g2["pa"], g0["pa"]) and np.array_equal(g2["pb"], g0["pb"])
         for key in ("limbs", "exp", "sign"):
             assert np.array_equal(g2["C"][key], g0["C"][key])
@@ -524,10 +527,10 @@ def _groups(moduli, req):
 
 
 @pytest.mark.parametrize("p,shape,req,kw", [
-    (256, (150, 130, 200), 20, {}),                 # CUDA-core residues, groups across the one/two-limb border
+    (256, (150, 130, 200), 20, {}),                 # residues in registers, groups across the one/two-limb border
     (256, (150, 130, 200), 7, {"res_engine": 2}),   # tensor-core residues, small groups
     (1024, (70, 60, 90), 40, {}),                   # tensor-core residues (automatic), an odd one-limb border
-    (1024, (70, 60, 90), 40, {"res_engine": 3}),    # the same groups on the CUDA cores
+    (1024, (70, 60, 90), 40, {"res_engine": 3}),    # the same groups by dp4a
     (113, (40, 300, 70), 3, {"crt_engine": 3}),     # one or three planes per group
 ])
 def test_planes_streamed_in_modulus_groups(ozk, p, shape, req, kw):
