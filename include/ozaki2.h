@@ -101,13 +101,14 @@ typedef struct {
   int schedule;   /* OZ2_SCHED_* */
   int timing;     /* nonzero: record per-stage CUDA events (ozaki2_last_timings) */
   int crt_engine; /* 0: automatic (default): engine 2 where the CRT accumulator needs more than
-                     20 32-bit digits (p above about 240), CUDA cores otherwise; 1: CRT column sums as an exact bf16
+                     20 32-bit digits (p above about 240), engine 3 otherwise; 1: CRT column sums as an exact bf16
                      GEMM on the tensor cores where 2L <= 256, the accumulator has <= 40 digits
-                     and the tables fit in shared memory (CUDA cores otherwise); 2: the column
+                     and the tables fit in shared memory (engine 3 otherwise); 2: the column
                      sums of any length as an exact bf16 GEMM on the tensor cores, written as
                      group sums to the workspace and finished on the CUDA cores, where
-                     32 <= L <= 448 and M N >= 128 (CUDA cores otherwise);
-                     3: the CRT on the CUDA cores only */
+                     32 <= L <= 448 and M N >= 128 (engine 3 otherwise);
+                     3: a lane or lanes per output, warp-level products of the bytes of M_l up to
+                     12 digits, 64-bit multiply-adds on the CUDA cores beyond */
   int res_engine; /* 0: automatic (default): engine 2 for integers of more than 72 bytes
                      (p above about 550), engine 3 otherwise; 1: residues as an exact bf16
                      GEMM of the bytes of a_hat with a table of centered 2^(8b) mod m on the
@@ -375,7 +376,7 @@ OZ2_API int ozaki2_last_timings(ozaki2_plan plan, float ms[5]);
 
 /* The CRT stage of the same execute split in two, in milliseconds: [0] the
    column sums on the tensor cores (crt_engine 2; about 0 where none ran),
-   [1] the rest (the finish from the group sums, or the whole CUDA-core CRT).
+   [1] the rest (the finish from the group sums, or the whole CRT of another engine).
    Synchronises on the recorded events. */
 OZ2_API int ozaki2_last_crt_split(ozaki2_plan plan, float ms[2]);
 

@@ -181,7 +181,7 @@ struct ProbHost {
   size_t off_e, off_f, off_pa, off_pb, off_u;   // workspace offsets
   int kind;                    // 0: limb output; 1: binary64 output
   bool skip_a, skip_b;         // planes of that side are written by the caller
-  int crt_mode;                // 0: CUDA-core CRT class crt_cls; 1: tensor-core CRT (class crt_cls);
+  int crt_mode;                // 0: a lane or lanes per output, class crt_cls; 1: tensor-core CRT (class crt_cls);
                                // 2: tensor-core sums to R digits, then the finish
   int crt_kpad, crt_npad, crt_np, crt_ngrp;
   int crt_qgrp;                // crt_mode 2: groups that the workspace has room for
@@ -435,8 +435,9 @@ static int res_table_key(ozaki2_plan_s* pl, int l0, int L, int L1, int nb, int k
 // Groups of 32 column sums that the workspace holds for `cols` formed columns:
 // whole chunks of the columns that two (or one, for chunks of 128 and more) of
 // the accumulator slots beside V take, kpad / 2 of the 512 TMEM columns.  The sums
-// kernel no longer runs in such chunks and forms cols / 32 groups; the workspace
-// of a shape stays what it was.
+// kernel no longer runs in such chunks and forms cols / 32 groups; the room beyond
+// those (at p = 2048 15 groups for 11) is not used.  It stays because the size of a
+// shape's workspace is checked against this rule (tests/test_host_abi.py).
 static int crt_workspace_groups(int kpad, int npad, int cols) {
   int cw = std::min(256, ((512 - kpad / 2) / 2) & ~31);
   if (cw < 128 && cw < npad) cw = std::min(256, (512 - kpad / 2) & ~31);
@@ -539,12 +540,14 @@ static int build_problem(ozaki2_plan_s* pl, int64_t M, int64_t N, int64_t K, int
                        crt_tc_smem_bytes(h.crt_cls, kpad, npad, L, 1) <= 227 * 1024;
     // automatic choice: the tensor-core sums above 20 accumulator digits
     // (measured at 1024^3: 0.238 vs 0.248 ms at 21 digits, 0.27 vs 0.33 at 25,
-    // 0.42 vs 0.67 at 33; 0.21 vs 0.18 at 17), the one-lane CUDA-core CRT below
+    // 0.42 vs 0.67 at 33; 0.21 vs 0.18 at 17), one lane per output below
     const bool want_mm = o.crt_engine == 2 || (o.crt_engine == 0 && h.D32 > 20);
     // sums of any length: fp32 column sums exact for 2L 127^2 < 2^24 (the u
-    // copies are boxes of 32 moduli x 128 outputs: at least that many)
-    const bool mm_ok = want_mm && 2 * L * 127 * 127 < (1 << 24) && L >= 32 && M * N >= 128 &&
-                       kpad / 2 + 2 * 32 <= 512;
+    // copies are boxes of 32 moduli x 128 outputs: at least that many; the bound
+    // on L, which the exact sums include, is above the 334 of the widest plans, whose
+    // formed columns fit, crt_mm_fits)
+    const bool mm_ok = want_mm && L <= 448 && L >= 32 && M * N >= 128;
+    static_assert(2 * 448 * 127 * 127 < (1 << 24), "column sums are exact");
     h.crt_mode = tc_ok ? 1 : (mm_ok ? 2 : 0);
     h.crt_kpad = kpad;
     h.crt_npad = h.crt_mode == 2 ? npad_mm : npad;

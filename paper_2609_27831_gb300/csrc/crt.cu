@@ -1040,8 +1040,8 @@ __device__ __forceinline__ uint32_t sub_chain(const uint32_t (&a)[N], const uint
 // each is one warp's serial work in the launch's tail: with one v_l and one row of
 // M_l in flight it stretched the finish of 1024^3 p = 2048 to 0.65 ms (0.32 so).
 // A function of its own and 64 digits at a time (all at once: 96 registers) keep
-// the common path at 72 registers, which p = 512 and 1024 need (0.182 and 0.205 ms
-// at 72 and 96, 1536 x 1093 outputs of p = 512).
+// the common path at 64 registers, which p = 512 and 1024 need (0.182 and 0.205 ms
+// at 64 and 96, 1531 x 1093 outputs of p = 512).
 __device__ __noinline__ void rebuild_digits(const ProbDev& P, const uint32_t* Mdig, const uint32_t* s_negP,
                                             int64_t sidx, uint32_t alpha, int src, uint32_t* Rv) {
   const int lane = threadIdx.x & 31, D = P.D32, L = P.L, DS = P.DS;

@@ -79,13 +79,12 @@ struct ProbDev {
   int32_t crt_gskip;     // crt_mode 2, long finish: groups of 32 Y columns below this one are not
                          // formed (the finish's fast form starts at it; stored group g is crt_gskip + g)
   int32_t DS;            // digit stride of the CRT tables (digits of the kernel class)
-  int32_t crt_mode;      // 0: CUDA-core CRT; 1: column sums on the tensor cores (one kernel);
+  int32_t crt_mode;      // 0: a lane or lanes per output; 1: column sums on the tensor cores (one kernel);
                          // 2: column sums on the tensor cores written as digits R, then the finish
   uint32_t* dbg_chat;    // optional: [M*N][D32+1] sign word + |c_hat| digits
   int32_t crt_kpad;      // tensor-core CRT: K = 2L padded to a multiple of 64
   int32_t crt_npad;      // tensor-core CRT: 7-bit pieces of S padded to a multiple of 16
   int32_t crt_np;        // tensor-core CRT: 7-bit pieces of S (columns of Y)
-  int32_t pad2;
   int64_t upitch;        // row pitch of u [L][upitch]: M*N rounded up to a multiple of 8
   int32_t res_mode;      // 0: residues in registers (warp-level products, dp4a beyond 72 bytes); 1: byte GEMM;
                          // 2: the byte GEMM, warp-specialised (bytes in TMEM, table streamed)
@@ -96,7 +95,6 @@ struct ProbDev {
   int32_t crt_ngrp;      // crt_mode 2: groups of 32 columns formed
   int32_t res_cw;        // res_mode 2: columns of Y per chunk (a multiple of 32)
   int32_t res_nchunk;    // res_mode 2: chunks
-  int32_t pad3;
   int32_t res_nabuf;     // res_mode 2: byte buffers (A) in TMEM (2 or 4)
   int32_t u_map;         // 1: tensor map 5 * count + i stores v_l tiles (N a multiple of 8)
   int32_t* dbg_prods;    // optional (K within one chunk): [G][M][N] exact plane sums before reduction

@@ -85,7 +85,7 @@ __device__ __forceinline__ uint32_t sig_word(const uint32_t* __restrict__ limbs3
   return __ldg(limbs32 + 2 * ((int64_t)(j >> 1) * ps + off) + (j & 1));
 }
 
-// Plane stores of the CUDA-core residues as global-space stores: the compiler
+// Plane stores of the dp4a residues as global-space stores: the compiler
 // then knows they cannot alias the shared-memory tables, and may read the next
 // modulus's table row ahead of them (about 1 % at 1024^3, p = 256).
 __device__ __forceinline__ void st_plane(uint16_t* p, uint32_t bits) { __stcg(reinterpret_cast<unsigned short*>(p), (unsigned short)bits); }
@@ -675,7 +675,7 @@ __global__ void __launch_bounds__(kRtThreads, 2)
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(s * tcols);
     auto centered_bits = [&](float rf, float mf) -> float {
       float x = (2.f * rf > mf) ? rf - mf : rf;      // (-m/2, m/2] of |a_hat| mod m
-      if (neg && x != 0.f) x = -x;                   // no -0: planes as the CUDA-core kernel
+      if (neg && x != 0.f) x = -x;                   // no -0: planes as the other kernels
       if (2.f * x == -mf) x = -x;                    // tie of the even modulus stays +m/2
       return x;
     };

@@ -149,13 +149,13 @@ def test_crt_sum_engine_workspace(ozk, p, cw_want):
     ngrp, up = -(-(npad - 32 * gskip) // cw) * cw // 32, 256 * 256
     a256 = lambda x: -(-x // 256) * 256
     assert plan.info["workspace_bytes"] - base["workspace_bytes"] == a256(4 * ngrp * 9 * up) + a256(4 * up)
-    small = (4, 4, 4, 53)                        # M N < 128: the CUDA-core CRT
+    small = (4, 4, 4, 53)                        # M N < 128: engine 3
     assert ozk.Plan(small, crt_engine=2).info["workspace_bytes"] == ozk.Plan(small, crt_engine=3).info["workspace_bytes"]
 
 
 def test_crt_engine_choice(ozk):
     """The automatic CRT choice: tensor-core sums where the accumulator needs
-    more than 20 digits; engine 3 keeps the CUDA cores; engine 2 asks for the
+    more than 20 digits, a lane or lanes per output (engine 3) below; engine 2 asks for the
     sums wherever the shape qualifies (L >= 32, M N >= 128)."""
     lo, mid, hi = (64, 64, 64, 200), (64, 64, 64, 384), (64, 64, 64, 1024)
     assert ozk.Plan(lo).info["crt_digits"] <= 20 and ozk.Plan(lo).info["crt_mode"] == 0
@@ -171,8 +171,8 @@ def test_crt_engine_choice(ozk):
 
 def test_residue_engine_choice(ozk):
     """The automatic residue choice: the warp-specialised tensor-core kernel for
-    integers of more than 72 bytes (t + 1 bits), the CUDA cores below; engine 3
-    forces the CUDA cores, engine 2 asks for the tensor cores up to 448 bytes."""
+    integers of more than 72 bytes (t + 1 bits), the register form below; engine 3
+    keeps out of the byte GEMM, engine 2 asks for it up to 448 bytes."""
     assert ozk.Plan((64, 64, 64, 2048)).info["res_mode"] == 2
     assert ozk.Plan((64, 64, 64, 1024)).info["res_mode"] == 2
     t = ozk.Plan((64, 64, 64, 553)).info["t"]
