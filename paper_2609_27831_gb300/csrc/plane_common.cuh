@@ -272,31 +272,46 @@ __device__ __forceinline__ void epi_chunk(const Job& j, const EpiConst& e, uint3
   }
 }
 
+// Outputs of up to kNarrow columns take the chunks that hold any of them: the others
+// cost as much as those, most of the stage for a few vectors (plane GEMMs with every
+// chunk and so, ms: 4578 x 2 x 89 p = 151 0.094 and 0.035, 673 x 4 x 34 p = 1798 0.157
+// and 0.057, 2000 x 60 x 500 p = 256 0.088 and 0.059).  Wider ones take all: leaving out
+// the last tile's gave 1531 x 1093 x 1777 p = 512 1.13 for 1.14, but 64 uneven products
+// 8.02 for 7.87.  A function of its own, so that the common loop keeps its code: eight
+// 1024 x 1024 x 64 p = 512 1.436 ms, 1.453 with the bound in that loop.
+constexpr int kNarrow = 128;
+static __device__ __noinline__ uint32_t epi_job_narrow(Job j, EpiConst e, uint32_t tbase, UStage us, int nc) {
+  uint32_t v[32];
+  for (int c = 0; c < nc; ++c) {
+    tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * c), v);
+    tc::tmem_ld_wait_regs(v);
+    epi_chunk(j, e, v, tbase + (uint32_t)(32 * c), 32 * c, us);
+  }
+  if (!j.last) tc::tmem_wait_st();
+  return us.n;
+}
+
 // The epilogue of one job over NC chunks of 32 columns at tbase, the TMEM
 // load of each chunk in flight while the one before it is reduced.  Ends
-// with every TMEM store of the job complete.  Outputs of up to kNarrow columns
-// take the chunks that hold any of them: the others cost as much as those, most of
-// the stage for a few vectors (plane GEMMs with every chunk and so, ms: 4578 x 2 x 89
-// p = 151 0.094 and 0.034, 673 x 4 x 34 p = 1798 0.157 and 0.057, 2000 x 60 x 500
-// p = 256 0.088 and 0.057).  Wider ones take all: leaving out the last tile's gave
-// 1531 x 1093 x 1777 p = 512 1.13 for 1.14, but 64 uneven products 8.02 for 7.87.
-constexpr int kNarrow = 128;
+// with every TMEM store of the job complete.
 template <int NC>
 __device__ __forceinline__ void epi_job(const Job& j, const EpiConst& e, uint32_t tbase, UStage& us) {
   static_assert(NC % 2 == 0, "chunks go in pairs");
-  const int nc = e.N <= kNarrow ? min(NC, (e.N - e.col0 + 31) >> 5) : NC;
-  if (nc <= 0) return;
+  if (e.N <= kNarrow) {
+    us.n = epi_job_narrow(j, e, tbase, us, min(NC, (e.N - e.col0 + 31) >> 5));
+    return;
+  }
   uint32_t va[32], vb[32];
   tc::tmem_ld32_nowait(tbase, va);
   tc::tmem_ld_wait_regs(va);
 #pragma unroll 1
-  for (int c = 0; c < nc; c += 2) {
+  for (int c = 0; c < NC; c += 2) {
     tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * (c + 1)), vb);
     epi_chunk(j, e, va, tbase + (uint32_t)(32 * c), 32 * c, us);
     tc::tmem_ld_wait_regs(vb);
-    if (c + 2 < nc) tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * (c + 2)), va);
-    if (c + 1 < nc) epi_chunk(j, e, vb, tbase + (uint32_t)(32 * (c + 1)), 32 * (c + 1), us);
-    if (c + 2 < nc) tc::tmem_ld_wait_regs(va);
+    if (c + 2 < NC) tc::tmem_ld32_nowait(tbase + (uint32_t)(32 * (c + 2)), va);
+    epi_chunk(j, e, vb, tbase + (uint32_t)(32 * (c + 1)), 32 * (c + 1), us);
+    if (c + 2 < NC) tc::tmem_ld_wait_regs(va);
   }
   if (!j.last) tc::tmem_wait_st();
 }
