@@ -29,6 +29,9 @@ def _allocator(device: torch.device, out: list) -> L.ALLOC_FN:
     return L.ALLOC_FN(alloc)
 
 
+_NO_ALLOCATOR = L.ALLOC_FN()                 # null: the library's memory
+
+
 class _Cache:
     """Owns one library cache handle (freed when the graph node dies) and the memory of its planes."""
 
@@ -61,8 +64,9 @@ class OzakiMatmul(torch.autograd.Function):
         need = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
         mem = []
         st = L.lib().ozaki2_dgemm_fwd_alloc(M, N, K, A.data_ptr(), K, B.data_ptr(), N, Cm.data_ptr(), N,
-                                            C.byref(opts) if opts is not None else None, _allocator(A.device, mem),
-                                            None, C.byref(h) if need else None,
+                                            C.byref(opts) if opts is not None else None,
+                                            _allocator(A.device, mem) if need else _NO_ALLOCATOR, None,
+                                            C.byref(h) if need else None,
                                             torch.cuda.current_stream(A.device).cuda_stream)
         L.check(st, "ozaki2_dgemm_fwd")
         ctx.cache = _Cache(h, mem[0]) if need else None
